@@ -260,29 +260,27 @@ int wf_launch_count(unsigned long long* n);
  *   shape[3]  lines per warp of the x passes (1, 2 or 4; at most 32 / chunks
  *             per line, which is also the default),
  *   shape[4]  lines per CTA of the second x pass,
- *   shape[5]  where Peaceman-Rachford with one F per step forms the right-hand
- *             side of its second x pass: 1 inside that pass (from staged rows
- *             of T* and F), 2 in a streaming matvec kernel before it (one more
- *             pass over R, but every thread busy on short lines);
- *   shape[6]  step form: 1 one launch per pass (seven or eight per step), 2 one
- *             persistent launch per step over every active slot (Peaceman-
- *             Rachford with one F per step, FP32, p <= 2, wind rank <= 2,
- *             no manufactured forcing; elsewhere the per-pass form runs),
- *             3 the per-pass launches over two groups of slots (the first
+ *   shape[5]  accepted and ignored (it placed the right-hand side of the second
+ *             x pass of Peaceman-Rachford with one F per step, whose combined
+ *             form has no second x pass);
+ *   shape[6]  step form: 0 one launch per direction (T and fuel side by
+ *             side), 1 Peaceman-Rachford with one F per step: one launch per
+ *             direction and array (seven per step in FP32; elsewhere as 0),
+ *             2 one persistent launch for the line passes of every active slot
+ *             (Peaceman-Rachford with one F per step; elsewhere as 0),
+ *             3 the launches of form 0 over two groups of slots (the first
  *             and the second half) on two streams, the second group's
  *             quadrature of a step starting when the first group's ends, so
  *             that one group's quadrature runs beside the other group's line
  *             passes; the groups join at the end of each wf_step call (and
  *             of each captured graph of steps).  Batches of two or more
  *             slots without manufactured forcing; profiled steps and
- *             wf_step_noalloc run the per-pass form;
+ *             wf_step_noalloc run the launches of form 1;
  *   shape[7]  slots per group of the persistent step's work order (the order
  *             keeps about six groups' fields live, sized for the L2 cache);
- * 0 selects the built-in rule (shape[5]: inside the pass; shape[6]: the
- * per-pass launches).
- * Every value changes the schedule only: both right-hand-side placements and
- * every step form perform the same operations in the same order, so the
- * results are the same bits.  wf_autotune tunes one value at a
+ * 0 selects the built-in rule.
+ * Every value changes the schedule only: every step form performs the same
+ * operations in the same order, so the results are the same bits.  wf_autotune tunes one value at a
  * time (two sweeps, the others held at their best values): each candidate
  * is timed in three rounds (the candidates in alternating order, so that a
  * drift of the clocks favours none), each round about reps steps (graphs
@@ -488,7 +486,7 @@ void wf_server_destroy(wf_server* s);
  * tables and factors; T and fuel are device arrays of Ny rows with a row pitch of
  * `pitch` >= Nx float elements, updated in place.  The intermediate fields of
  * the step live in one static device array that the library reserves on every
- * GPU it is loaded on (6 MiB, held until the process exits); pitch * Ny must not
+ * GPU it is loaded on (4 MiB, held until the process exits); pitch * Ny must not
  * exceed 524288 (512 x 512 elements of degree 2 fit).  The first call on a
  * device looks up that array's device address; make that first call before any
  * stream capture.  All calls share the array: two calls whose work overlaps on

@@ -79,9 +79,9 @@ struct Slot {
     double coef[2][3][3] = {};  // [dir][op][aM, aK, aG]
 };
 
-enum SiteId { S_RHS1, S_X1, S_Y1, S_Y2PRE, S_RHS2, S_MV2, S_X2, S_Y3, S_PERSIST, S_NSITES };
+enum SiteId { S_RHS1, S_X1, S_Y1, S_Y2PRE, S_RHS2, S_X2, S_Y3, S_PERSIST, S_NSITES };
 const char* kSiteNames[S_NSITES] = {"rhs_quadrature_1", "xsolve_1", "ysolve_1", "ysolve_y_substep",
-                                    "rhs_quadrature_2", "matvec_2", "xsolve_2", "ysolve_2",
+                                    "rhs_quadrature_2", "xsolve_2", "ysolve_2",
                                     "step_persistent"};
 
 }  // namespace
@@ -131,10 +131,9 @@ struct wf_handle {
     double* tdev = nullptr;    // device: start time of the next step (advanced only with forcing)
     int tune[kTune] = {0, 0, 0, 0, 0, 0, 0, 0};  // x lines per CTA (first x pass), y lines per CTA,
                                            // quadrature segment rows, x lines per warp, x lines
-                                           // per CTA of the second x pass, its right-hand side
-                                           // (1 fused, 2 separate matvec), step form (1 per-pass
-                                           // launches, 2 persistent), slots per group of the
-                                           // persistent order (0: the launchers' rules)
+                                           // per CTA of the second x pass, unused, step form
+                                           // (wf_set_tuning), slots per group of the persistent
+                                           // order (0: the launchers' rules)
     // persistent step: work items, ticket / abort / item count, arrival counters (allocated on
     // first use); the item list is rebuilt when the active slots or the shapes change
     int4* p_items = nullptr;
@@ -143,7 +142,7 @@ struct wf_handle {
     size_t p_items_cap = 0, p_cnt_cap = 0;
     bool p_dirty = true;
     bool noalloc_run = false;  // wf_step_noalloc in progress: per-pass launches only
-    void *T = nullptr, *phi = nullptr, *F = nullptr, *Phi = nullptr, *R = nullptr;
+    void *T = nullptr, *phi = nullptr, *Phi = nullptr, *R = nullptr;
     int* status = nullptr;
     void *fxq = nullptr, *gxq = nullptr, *fyq = nullptr, *gyq = nullptr;
     std::vector<Slot> slots;
@@ -252,7 +251,6 @@ void layout_slot(wf_handle* h, Arena& A) {
     const size_t field = (size_t)h->Ny * h->pitch;
     h->T = A.take<char>(field * es);
     h->phi = A.take<char>(field * es);
-    h->F = A.take<char>(field * es);
     h->Phi = A.take<char>(field * es);
     h->R = A.take<char>(field * es);
     h->status = A.take<int>(4);
@@ -598,8 +596,17 @@ cudaError_t upload_active(wf_handle* h) {
 // Every substep is solved for its increment: with X_+ = M + theta A_x and
 // Y_+ = M + theta A_y, the PR systems of Eq. matrixPR are identical to
 //   (X_+ (x) M^y) (T* - T^n)      = theta F - theta (A_x (x) M^y) T^n - theta (M^x (x) A_y) T^n
-//   (M^x (x) Y_+) (T^{n+1} - T*)  = theta F - theta (A_x (x) M^y) T*  - theta (M^x (x) A_y) T*
-// and the Strang/Crank-Nicolson systems of Eq. matrixCN to
+//   (M^x (x) Y_+) (T^{n+1} - T*)  = theta F* - theta (A_x (x) M^y) T*  - theta (M^x (x) A_y) T*
+// With one F per step (F* = F) the intermediate T* drops out.  Write B_x = (M^x)^{-1} A_x,
+// B_y = (M^y)^{-1} A_y, G = (M^x (x) M^y)^{-1} F and W = (I - theta B_y) T^n + theta G: substep 1 is
+// (I + theta B_x) T* = W, so (I - theta B_x) T* = 2 T* - W, and substep 2 becomes
+// (I + theta B_y) T^{n+1} = 2 T* - (I - theta B_y) T^n, that is
+// (I + theta B_y) (T^{n+1} - T^n) = 2 (T* - T^n), or
+//   (X_+ (x) Y_+) (T^{n+1} - T^n) = tau F - tau (A_x (x) M^y) T^n - tau (M^x (x) A_y) T^n:
+// the same T^{n+1} from one right-hand side, one x and one y solve.  Against forming T* (a second
+// right-hand side, x solve and y solve; default launch shapes) the step of 256 scenarios of 258^2 coefficients went from
+// 854 to 564 us, of one 4099^2 cubic domain from 4291 to 896 us.
+// The Strang/Crank-Nicolson systems of Eq. matrixCN to
 //   (X_+ (x) M^y) (T* - T^n)      = tau/2 F(T^n) - 2 theta_x (A_x (x) M^y) T^n        (theta_x = tau/4)
 //   (I (x) Y_+) (T** - T*)        = -2 theta_y (I (x) A_y) T*                         (theta_y = tau/2)
 //   (X_+ (x) M^y) (T^{n+1} - T**) = tau/2 F(T**) - 2 theta_x (A_x (x) M^y) T**
@@ -633,36 +640,16 @@ void persist_args(wf_handle* h, PersistHost* ph) {
     Op* Y = h->dy.op;
     const Chunks& cx = h->dx.ch;
     const Chunks& cy = h->dy.ch;
-    const double th = 0.5 * h->dt;
     memset(ph, 0, sizeof(*ph));
     ph->prec = h->prec;
     ph->p = h->p;
-    ph->x1 = line_args(h, 1);
-    add_line(ph->x1, h->R, h->R, X[2], cx);
-    add_line(ph->x1, h->Phi, h->Phi, X[0], cx);
-    ph->y1 = line_args(h, 0);
-    add_line(ph->y1, h->R, h->T, Y[0], cy, h->T);
-    add_line(ph->y1, h->Phi, h->phi, Y[0], cy, h->phi);
-    MatvecArgs& mv = ph->mv;
-    mv.Nx = h->Nx;
-    mv.Ny = h->Ny;
-    mv.pitch = h->pitch;
-    mv.T = h->T;
-    mv.F = h->F;
-    mv.R = h->R;
-    mv.A1 = X[1].bandP;
-    mv.B1 = Y[0].bandP;
-    mv.A2 = X[0].bandP;
-    mv.B2 = Y[1].bandP;
-    mv.Fscale = th;
-    mv.c1 = 1.0;
-    mv.c2 = 1.0;
-    mv.b = batch(h);
-    ph->x2 = line_args(h, 2);
-    add_line(ph->x2, h->R, h->R, X[0], cx);
-    ph->y2 = line_args(h, 0);
-    add_line(ph->y2, h->R, h->T, Y[2], cy, h->T);
-    ph->y2.status = h->status;
+    ph->x = line_args(h, 1);
+    add_line(ph->x, h->R, h->R, X[2], cx);
+    add_line(ph->x, h->Phi, h->Phi, X[0], cx);
+    ph->y = line_args(h, 0);
+    add_line(ph->y, h->R, h->T, Y[2], cy, h->T);
+    add_line(ph->y, h->Phi, h->phi, Y[0], cy, h->phi);
+    ph->y.status = h->status;
     ph->xG = h->tune[0];
     ph->yG = h->tune[1];
     ph->nslots_cap = h->S;
@@ -704,7 +691,7 @@ int prepare_persist(wf_handle* h) {
         if (h->active_host[z]) act.push_back(z);
     // room for every slot active, so that slots joining later need no reallocation
     // at most one item per tile
-    const size_t most = (size_t)plan.narr1 * (plan.nxg + plan.nyg) + (plan.nmv + 7) / 8 + plan.nxg + plan.nyg;
+    const size_t most = (size_t)plan.narr * (plan.nxg + plan.nyg);
     const size_t cap = std::max<size_t>(1, (size_t)h->S * most);
     const size_t need_cnt = (size_t)h->S * plan.cstride;
     if (cap > h->p_items_cap || need_cnt > h->p_cnt_cap || !h->p_ctl) {
@@ -825,22 +812,41 @@ cudaError_t enqueue_step_body(wf_handle* h) {
         if ((e = timed(h, S_Y3, [&] { return launch_ysolve(prec, p, y1, s); })) != cudaSuccess) return e;
         return cudaSuccess;
     }
-    if (h->prm.scheme == WF_PR && use_persist(h) && h->p_ctl) {
-        // the quadrature (and forcing) as in the per-pass form, then one launch for the rest
-        const double th = 0.5 * h->dt;
-        RhsArgs r1 = rhs_args(h, h->T, h->F, h->Phi, h->R, th, X[1], Y[0], 1.0, &X[0], &Y[1], 1.0);
-        r1.single = 1;  // the quadrature in one launch: two launches per step in all
-        auto l1 = [&] { return rhs_and_forcing(h, r1, h->R, th, h->F, 1.0); };
+    if (h->prm.scheme == WF_PR && h->prm.F_timing == WF_F_ONCE) {
+        // R = tau F + 2 (op1_x (x) M^y) T + 2 (M^x (x) op1_y) T, then X_+ lines along x, Y_+ along y
+        RhsArgs r1 = rhs_args(h, h->T, nullptr, h->Phi, h->R, h->dt, X[1], Y[0], 2.0, &X[0], &Y[1], 2.0);
+        const bool pers = use_persist(h) && h->p_ctl;
+        r1.single = pers ? 1 : 0;  // the quadrature in one launch: two launches per step in all
+        auto l1 = [&] { return rhs_and_forcing(h, r1, h->R, h->dt, nullptr, 0.0); };
         if ((e = timed(h, S_RHS1, l1)) != cudaSuccess) return e;
-        PersistHost ph;
-        persist_args(h, &ph);
-        return timed(h, S_PERSIST, [&] { return persist_step(ph, nullptr, true, s); });
+        if (h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return e;
+        if (pers) {
+            PersistHost ph;
+            persist_args(h, &ph);
+            return timed(h, S_PERSIST, [&] { return persist_step(ph, nullptr, true, s); });
+        }
+        // both arrays in one launch per direction; step form 1: a launch per array
+        const bool split = h->tune[6] == 1 || (h->tune[6] == 3 && h->gn == 0);
+        for (int part = 0; part < (split ? 2 : 1); ++part) {
+            LineArgs x1 = line_args(h, 1);
+            if (part == 0) add_line(x1, h->R, h->R, X[2], cx);
+            if (part == 1 || !split) add_line(x1, h->Phi, h->Phi, X[0], cx);
+            if ((e = timed(h, S_X1, [&] { return launch_xsolve(prec, p, x1, s); })) != cudaSuccess) return e;
+        }
+        for (int part = 0; part < (split ? 2 : 1); ++part) {
+            LineArgs y1 = line_args(h, 0);
+            if (part == 0) add_line(y1, h->R, h->T, Y[2], cy, h->T);
+            if (part == 1 || !split) add_line(y1, h->Phi, h->phi, Y[0], cy, h->phi);
+            if (part == 0) y1.status = h->status;  // the guard watches T
+            if ((e = timed(h, S_Y1, [&] { return launch_ysolve(prec, p, y1, s); })) != cudaSuccess) return e;
+        }
+        return cudaSuccess;
     }
     if (h->prm.scheme == WF_PR) {
+        // F re-evaluated at T* in the second substep
         const double th = 0.5 * h->dt;
-        const bool once = h->prm.F_timing == WF_F_ONCE;
-        RhsArgs r1 = rhs_args(h, h->T, once ? h->F : nullptr, h->Phi, h->R, th, X[1], Y[0], 1.0, &X[0], &Y[1], 1.0);
-        auto l1 = [&] { return rhs_and_forcing(h, r1, h->R, th, once ? h->F : nullptr, 1.0); };
+        RhsArgs r1 = rhs_args(h, h->T, nullptr, h->Phi, h->R, th, X[1], Y[0], 1.0, &X[0], &Y[1], 1.0);
+        auto l1 = [&] { return rhs_and_forcing(h, r1, h->R, th, nullptr, 0.0); };
         if ((e = timed(h, S_RHS1, l1)) != cudaSuccess) return e;
         if (h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return e;
         LineArgs x1 = line_args(h, 1);
@@ -849,57 +855,16 @@ cudaError_t enqueue_step_body(wf_handle* h) {
         if ((e = timed(h, S_X1, [&] { return launch_xsolve(prec, p, x1, s); })) != cudaSuccess) return e;
         LineArgs y1 = line_args(h, 0);
         add_line(y1, h->R, h->T, Y[0], cy, h->T);
-        if (once) add_line(y1, h->Phi, h->phi, Y[0], cy, h->phi);
         if ((e = timed(h, S_Y1, [&] { return launch_ysolve(prec, p, y1, s); })) != cudaSuccess) return e;
-        bool fused = false;
-        if (once && h->tune[5] != 2) {
-            // substep 2 in one x pass: R = th F + (op1_x (x) M^y) T* + (M^x (x) op1_y) T*, then M^x lines
-            LineArgs x2 = line_args(h, 2);
-            add_line(x2, nullptr, h->R, X[0], cx);
-            x2.preT = h->T;
-            x2.preF = h->F;
-            x2.preFscale = th;
-            x2.pc1 = 1.0;
-            x2.pc2 = 1.0;
-            x2.pA1 = X[1].bandP;
-            x2.pB1 = Y[0].bandP;
-            x2.pA2 = X[0].bandP;
-            x2.pB2 = Y[1].bandP;
-            e = timed(h, S_X2, [&] { return launch_xsolve(prec, p, x2, s); });
-            if (e == cudaSuccess) fused = true;
-            else if (e != cudaErrorNotSupported) return e;
-            else cudaGetLastError();
-        }
-        if (once && !fused) {
-            MatvecArgs mv;
-            mv.Nx = h->Nx;
-            mv.Ny = h->Ny;
-            mv.pitch = h->pitch;
-            mv.T = h->T;
-            mv.F = h->F;
-            mv.R = h->R;
-            mv.A1 = X[1].bandP;
-            mv.B1 = Y[0].bandP;
-            mv.A2 = X[0].bandP;
-            mv.B2 = Y[1].bandP;
-            mv.Fscale = th;
-            mv.c1 = 1.0;
-            mv.c2 = 1.0;
-            mv.b = batch(h);
-            if ((e = timed(h, S_MV2, [&] { return launch_matvec(prec, p, mv, s); })) != cudaSuccess) return e;
-        } else if (!once) {
-            RhsArgs r2 = rhs_args(h, h->T, nullptr, nullptr, h->R, th, X[1], Y[0], 1.0, &X[0], &Y[1], 1.0);
-            auto l2 = [&] { return rhs_and_forcing(h, r2, h->R, th, nullptr, 0.0); };
-            if ((e = timed(h, S_RHS2, l2)) != cudaSuccess) return e;
-        }
-        if (!fused) {
-            LineArgs x2 = line_args(h, 2);
-            add_line(x2, h->R, h->R, X[0], cx);
-            if ((e = timed(h, S_X2, [&] { return launch_xsolve(prec, p, x2, s); })) != cudaSuccess) return e;
-        }
+        RhsArgs r2 = rhs_args(h, h->T, nullptr, nullptr, h->R, th, X[1], Y[0], 1.0, &X[0], &Y[1], 1.0);
+        auto l2 = [&] { return rhs_and_forcing(h, r2, h->R, th, nullptr, 0.0); };
+        if ((e = timed(h, S_RHS2, l2)) != cudaSuccess) return e;
+        LineArgs x2 = line_args(h, 2);
+        add_line(x2, h->R, h->R, X[0], cx);
+        if ((e = timed(h, S_X2, [&] { return launch_xsolve(prec, p, x2, s); })) != cudaSuccess) return e;
         LineArgs y2 = line_args(h, 0);
         add_line(y2, h->R, h->T, Y[2], cy, h->T);
-        if (!once) add_line(y2, h->Phi, h->phi, Y[0], cy, h->phi);
+        add_line(y2, h->Phi, h->phi, Y[0], cy, h->phi);
         y2.status = h->status;
         if ((e = timed(h, S_Y3, [&] { return launch_ysolve(prec, p, y2, s); })) != cudaSuccess) return e;
         return cudaSuccess;
@@ -1710,8 +1675,7 @@ int wf_autotune(wf_handle* h, int reps) {
     static const int kSeg[] = {0, 128, 96, 80, 64, 56, 48, 40, 32, 28, 24, 21, 20, 16, 12};
     static const int kLines[] = {0, 32, 16, 8, 4, 2, 1};
     static const int kRpw[] = {0, 1, 2, 4};
-    static const int kFuse[] = {0, 2};
-    static const int kModeAll[] = {1, 2, 3};  // per-pass, persistent, per-pass in two slot groups
+    static const int kModeAll[] = {0, 2, 3};  // the rule, persistent, two slot groups
     static const int kGroup[] = {0, 1, 2, 4, 8, 16, 32, 64};
     struct Axis {
         int q;
@@ -1721,17 +1685,19 @@ int wf_autotune(wf_handle* h, int reps) {
     const bool pers = persist_supported(h->prec, h->p, h->wr) && h->prm.scheme == WF_PR &&
                       h->prm.F_timing == WF_F_ONCE;
     const bool grp = h->S >= 2 && !h->mms_on;
+    // only Strang / Crank-Nicolson and F per substep have a second x pass
+    const bool second_x = h->prm.scheme == WF_STRANG_CN ||
+                          (h->prm.scheme == WF_PR && h->prm.F_timing == WF_F_PER_SUBSTEP);
     int kMode[3], nMode = 0;
     for (int m : kModeAll)
-        if (m == 1 || (m == 2 && pers) || (m == 3 && grp)) kMode[nMode++] = m;
-    // the shapes first (in the per-pass form, the rule), then the step form with those shapes and
+        if (m == 0 || (m == 2 && pers) || (m == 3 && grp)) kMode[nMode++] = m;
+    // the shapes first (in the rule's form), then the step form with those shapes and
     // the persistent form's group size; the second sweep refines the shapes under the chosen form
     const Axis order[] = {{2, kSeg, (int)(sizeof(kSeg) / sizeof(int))},
                           {0, kLines, (int)(sizeof(kLines) / sizeof(int))},
                           {3, kRpw, (int)(sizeof(kRpw) / sizeof(int))},
                           {1, kLines, (int)(sizeof(kLines) / sizeof(int))},
-                          {4, kLines, (int)(sizeof(kLines) / sizeof(int))},
-                          {5, kFuse, (int)(sizeof(kFuse) / sizeof(int))},
+                          {4, kLines, second_x ? (int)(sizeof(kLines) / sizeof(int)) : 0},
                           {6, kMode, nMode > 1 ? nMode : 0},
                           {7, kGroup, pers && h->S > 1 ? (int)(sizeof(kGroup) / sizeof(int)) : 0}};
     const size_t bytes = (size_t)h->sbytes * h->S;
@@ -1906,13 +1872,13 @@ int wf_set_tuning(wf_handle* h, const int* shape) {
 
 // ---- allocation-free step ------------------------------------------------------------
 //
-// Scratch of wf_step_noalloc: the three intermediate fields of a step (F, Phi, R), each at
+// Scratch of wf_step_noalloc: the two intermediate fields of a step (Phi, R), each at
 // most kNoallocMaxElems padded FP32 coefficients, in one array that every GPU loading
-// this library holds until the process exits (6 MiB).  Host code must not hand the
+// this library holds until the process exits (4 MiB).  Host code must not hand the
 // symbol itself to a kernel: on the host it names a host-side placeholder.  Its device
 // address is looked up once per device with cudaGetSymbolAddress and cached.
 constexpr size_t kNoallocMaxElems = size_t(1) << 19;
-static __device__ __align__(256) float g_noalloc_scratch[3 * kNoallocMaxElems];
+static __device__ __align__(256) float g_noalloc_scratch[2 * kNoallocMaxElems];
 
 namespace {
 constexpr int kNoallocMaxDevices = 64;
@@ -1952,13 +1918,12 @@ extern "C" int wf_step_noalloc(wf_handle* h, void* T, void* fuel, int pitch, int
     // Run the handle's own step sequence with the caller's state and the static scratch in
     // place of the handle's buffers.  Every scratch element a kernel reads was written earlier
     // in the same step, so nothing needs clearing between calls.
-    void* save[5] = {h->T, h->phi, h->F, h->Phi, h->R};
+    void* save[4] = {h->T, h->phi, h->Phi, h->R};
     const int save_pitch = h->pitch;
     h->T = T;
     h->phi = fuel;
-    h->F = scratch;
-    h->Phi = scratch + kNoallocMaxElems;
-    h->R = scratch + 2 * kNoallocMaxElems;
+    h->Phi = scratch;
+    h->R = scratch + kNoallocMaxElems;
     h->pitch = pitch;
     cudaError_t e = cudaSuccess;
     h->noalloc_run = true;  // the persistent step's buffers may not exist yet: per-pass launches
@@ -1966,9 +1931,8 @@ extern "C" int wf_step_noalloc(wf_handle* h, void* T, void* fuel, int pitch, int
     h->noalloc_run = false;
     h->T = save[0];
     h->phi = save[1];
-    h->F = save[2];
-    h->Phi = save[3];
-    h->R = save[4];
+    h->Phi = save[2];
+    h->R = save[3];
     h->pitch = save_pitch;
     return e == cudaSuccess ? WF_OK : WF_ECUDA;
 }

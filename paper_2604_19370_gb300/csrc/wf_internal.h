@@ -186,7 +186,7 @@ cudaError_t launch_forcing(int prec, const MmsArgs& a, void* out1, double s1, vo
                            cudaStream_t s);
 cudaError_t launch_advance_time(double* t, double dt, cudaStream_t s);
 
-// ---- line solves and matvec (wf_solve.cu) -------------------------------------------
+// ---- line solves (wf_solve.cu) -------------------------------------------
 struct LineArgs {
     int G;       // lines per CTA of the compact-factor kernels (0: the launcher's rule; else an upper bound)
     int rpw;     // x pass: lines per warp (0: as many as the chunks allow; 1, 2: at most that many)
@@ -205,13 +205,7 @@ struct LineArgs {
                             // as scratch)
     long long wait_ns;      // limit of a bounded device wait (ns of %globaltimer; 0: give up at once)
     double tmax;
-    Batch b;  // per scenario: in, out, factors, premul, base, status, pre*
-    // x pass only, one array: when preT is set the input line is formed in the kernel as
-    // R = preFscale preF + pc1 (pA1 (x) pB1) preT + pc2 (pA2 (x) pB2) preT  (in[0] unused)
-    const void* preT;
-    const void* preF;
-    double preFscale, pc1, pc2;
-    const void *pA1, *pB1, *pA2, *pB2;
+    Batch b;  // per scenario: in, out, factors, premul, base, status
 };
 cudaError_t launch_xsolve(int prec, int p, const LineArgs& a, cudaStream_t s);
 cudaError_t launch_ysolve(int prec, int p, const LineArgs& a, cudaStream_t s);
@@ -237,26 +231,13 @@ size_t fac_pad_elems(int p, int mmax);
 cudaError_t launch_pad_factors(int prec, int p, int mmax, const void* luc, const void* spkc, const void* Ec,
                                void* fpad, cudaStream_t s);
 
-// R = Fscale F + c1 (A1 (x) B1) T + c2 (A2 (x) B2) T   (A2 may be NULL)
-struct MatvecArgs {
-    int Nx, Ny, pitch;
-    const void* T;
-    const void* F;
-    void* R;
-    const void *A1, *B1, *A2, *B2;
-    double Fscale, c1, c2;
-    Batch b;  // per scenario: every pointer
-};
-cudaError_t launch_matvec(int prec, int p, const MatvecArgs& a, cudaStream_t s);
-
 // ---- persistent line passes (wf_persist.cu) -----------------------------------------
 // After the quadrature launch of a Peaceman-Rachford step (one F per step), one launch runs the
-// step's x, y and matvec passes for every active slot, over the (pass, slot, tile) items listed
+// step's x and y passes for every active slot, over the (pass, slot, tile) items listed
 // by persist_items; the arguments are those of the per-pass launches of the same step.
 struct PersistHost {
     int prec, p;
-    LineArgs x1, y1, x2, y2;  // x1 and y1 with two arrays (R, Phi), x2 and y2 with one
-    MatvecArgs mv;            // substep-2 right-hand side
+    LineArgs x, y;            // two arrays each (R, Phi)
     int xG, yG;               // x lines and y columns per tile (0: rule)
     int nslots_cap;           // slot capacity of the handle (counter blocks)
     long long wait_ns;
@@ -269,7 +250,7 @@ struct PersistHost {
     int* budget;              // device: per-slot step budgets, or NULL (a spent budget, 0, skips too)
 };
 struct PersistPlan {
-    int nq, nmv, nxg, nyg, narr1, cstride, ctas, seg, xG, yG;
+    int nxg, nyg, narr, cstride, ctas;
     size_t smem;
 };
 bool persist_supported(int prec, int p, int wind_rank);

@@ -13,7 +13,6 @@ struct FastArgs {
     int nlines, pitch, mpad, G;
     int lsh;  // x pass: log2 of the lanes per line (5: one line per warp; 4: two; 3: four)
     int sp;   // x pass: row stride of the staged rows in shared memory (elements)
-    int tsp;  // x pass with preT: row stride of the staged T* rows (data at column offset 4)
     Chunks ch;
     const P* in[2];
     P* out[2];
@@ -30,10 +29,6 @@ struct FastArgs {
     P tmax;
     int tma;  // x pass: rows staged with bulk copies (16-byte aligned rows)
     Batch b;
-    const P* preT;
-    const P* preF;
-    P preFscale, pc1, pc2;
-    const P *pA1, *pB1, *pA2, *pB2;
 };
 
 // Pointers of one array (blockIdx.y) of one scenario (blockIdx.z).  They are selected with
@@ -49,7 +44,6 @@ struct LineView {
     const P *luc, *spkc, *Ec, *fpad;
     int* status;
     int* tstatus;
-    const P *preT, *preF, *pA1, *pB1, *pA2, *pB2;
 };
 
 template <typename P>
@@ -67,12 +61,6 @@ __device__ __forceinline__ LineView<P> scene_line(const FastArgs<P>& a, int arr)
     v.fpad = scene_ptr(one ? a.fpad[1] : a.fpad[0], a.b);
     v.status = scene_ptr(a.status, a.b);
     v.tstatus = scene_ptr(a.tstatus, a.b);
-    v.preT = scene_ptr(a.preT, a.b);
-    v.preF = scene_ptr(a.preF, a.b);
-    v.pA1 = scene_ptr(a.pA1, a.b);
-    v.pB1 = scene_ptr(a.pB1, a.b);
-    v.pA2 = scene_ptr(a.pA2, a.b);
-    v.pB2 = scene_ptr(a.pB2, a.b);
     return v;
 }
 

@@ -1,5 +1,4 @@
-// Chunked line solves (TMA-staged x pass, column-parallel y pass) and the streaming Kronecker
-// matvec.
+// Chunked line solves (TMA-staged x pass, column-parallel y pass).
 //
 // Paper: Sec. 4 ("Cost of directional implicit solves"): each directional system
 // is a set of independent banded 1-D solves (half-bandwidth p) along x or y.
@@ -29,9 +28,8 @@ namespace {
 // (C <= lanes per line).
 // The G rows are contiguous in memory: one bulk copy stages them, one bulk store writes them back.
 // Chunk lengths are odd, so the 32 lanes of a warp read 32 distinct shared-memory banks.
-template <typename P, int PD, bool PRE>
+template <typename P, int PD>
 __global__ void __launch_bounds__(256) k_xsolve_warp(const FastArgs<P> a) {
-    constexpr int W = 2 * PD + 1;
     if (!scene_active(a.b)) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -44,36 +42,16 @@ __global__ void __launch_bounds__(256) k_xsolve_warp(const FastArgs<P> a) {
     const int rows = min(G, a.nlines - j0);
     const size_t row_bytes = (size_t)a.pitch * sizeof(P);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
-    constexpr bool pre = PRE;
     const int sp = a.sp;                                           // shared-memory row stride
     P* rowbuf = reinterpret_cast<P*>(smem_raw + 128);             // [G][sp]
-    // pre: T* rows j0-p .. j0+G+p-1 at stride tsp, values at column offset HO, zero halo columns
-    // on either side so that the column sweep needs no bounds checks
-    constexpr int HO = 4;
-    const int tsp = a.tsp;
-    P* tbuf = rowbuf + (size_t)G * sp;
-    const FacSmem<P, PD> fm(tbuf + (pre ? (size_t)(G + 2 * PD) * tsp : 0), mmax);  // factors, then pre: bands
-    const P* __restrict__ in = pre ? v.preF : v.in;
+    const FacSmem<P, PD> fm(rowbuf + (size_t)G * sp, mmax);
+    const P* __restrict__ in = v.in;
     P* out = v.out;
-    // rows of the halo block that exist (pre): lo .. hi-1
-    const int lo = max(0, j0 - PD), hi = min(a.nlines, j0 + rows + PD);
-
     // factors: one bulk copy of the operator's padded block beside the rows, else staged element
     // by element
     const bool fbulk = a.tma && v.fpad != nullptr;
     const uint32_t fbytes = (uint32_t)(fac_elems<PD>(mmax) * sizeof(P));
     bool staged = true;
-    if (pre) {
-        // halo rows outside the domain read as zero; so do the PD columns left of every row
-        for (int r = j0 - PD; r < j0 + rows + PD; ++r) {
-            P* row = tbuf + (size_t)(r - (j0 - PD)) * tsp;
-            if (r >= lo && r < hi) {
-                if (tid < PD) row[HO - PD + tid] = P(0);
-            } else {
-                for (int x = tid; x < tsp; x += blockDim.x) row[x] = P(0);
-            }
-        }
-    }
     if (a.tma) {
         // one bulk copy per row (the shared-memory stride differs from the global pitch);
         // thread 0 arms the barrier with the total, the lanes of warp 0 issue the copies
@@ -81,37 +59,20 @@ __global__ void __launch_bounds__(256) k_xsolve_warp(const FastArgs<P> a) {
             mbar_init(bar, 1);
             mbar_fence_init();
             const uint32_t bytes = (uint32_t)(rows * row_bytes);
-            const uint32_t tbytes = pre ? (uint32_t)((hi - lo) * row_bytes) : 0u;
-            mbar_expect_tx(bar, bytes + tbytes + (fbulk ? fbytes : 0u));
+            mbar_expect_tx(bar, bytes + (fbulk ? fbytes : 0u));
         }
         __syncwarp();
         if (warp == 0) {
             if (fbulk && lane == 31) bulk_load(fm.F, v.fpad, fbytes, bar);
             for (int r = lane; r < rows; r += 32)
                 bulk_load(rowbuf + (size_t)r * sp, in + (size_t)(j0 + r) * a.pitch, (uint32_t)row_bytes, bar);
-            if (pre)
-                for (int r = lo + lane; r < hi; r += 32)
-                    bulk_load(tbuf + (size_t)(r - (j0 - PD)) * tsp + HO, v.preT + (size_t)r * a.pitch,
-                              (uint32_t)row_bytes, bar);
         }
     } else {
         for (int r = 0; r < rows; ++r)
             for (int x = tid; x < N; x += blockDim.x) rowbuf[(size_t)r * sp + x] = in[(size_t)(j0 + r) * a.pitch + x];
-        if (pre)
-            for (int r = lo; r < hi; ++r)
-                for (int x = tid; x < N; x += blockDim.x)
-                    tbuf[(size_t)(r - (j0 - PD)) * tsp + HO + x] = v.preT[(size_t)r * a.pitch + x];
     }
     if (!fbulk) stage_factors<P, PD>(v, mmax, fm);
-    if (pre) {
-        P* bco = fm.end();
-        for (int i = tid; i < rows * W; i += blockDim.x) {
-            const int r = i / W, d = i - r * W;
-            bco[(size_t)r * 2 * W + d] = a.pc1 * v.pB1[(size_t)(j0 + r) * W + d];
-            bco[(size_t)r * 2 * W + W + d] = v.pA2 ? a.pc2 * v.pB2[(size_t)(j0 + r) * W + d] : P(0);
-        }
-    }
-    __syncthreads();  // mbarrier initialised, factors staged, halo zeroed
+    __syncthreads();  // mbarrier initialised, factors staged
     if (a.tma) staged = mbar_wait_bounded(bar, 0, a.wait_ns);
     staged = __syncthreads_and(staged);  // one decision for the whole CTA (barriers follow)
     if (!staged) {
@@ -121,94 +82,6 @@ __global__ void __launch_bounds__(256) k_xsolve_warp(const FastArgs<P> a) {
         if (tid == 0 && v.tstatus) atomicOr(v.tstatus, 4);
         return;
     }
-    if (pre) {
-        // the PD columns right of every staged row read as zero (they may hold row padding)
-        for (int r = lo; r < hi; ++r)
-            if (tid < PD) tbuf[(size_t)(r - (j0 - PD)) * tsp + HO + N + tid] = P(0);
-        __syncthreads();
-        // R = preFscale F + (pA1 (x) pc1 pB1) T + (pA2 (x) pc2 pB2) T.  Work item = one column and
-        // a group of rh output rows: the x bands of the column are loaded once and applied to the
-        // rh + 2p staged rows the group needs, whose results pass through a W-row register window
-        // that the y bands reduce.  The number of row groups nh balances N * nh items over the
-        // CTA's threads against the 2p rows each group re-reads.
-        const P* __restrict__ bco = fm.end();  // [G][2][W], scaled by pc1 / pc2
-        const int nt = blockDim.x;
-        int nh = 1, rh = rows;
-        long best;
-        {
-            best = (long)((N + nt - 1) / nt) * (rows + 2 * PD);
-            for (int cand = 2; cand <= 8 && cand <= rows; cand *= 2) {
-                const int h = (rows + cand - 1) / cand;
-                const long cost = (long)((N * cand + nt - 1) / nt) * (h + 2 * PD);
-                if (cost < best) {
-                    best = cost;
-                    nh = cand;
-                    rh = h;
-                }
-            }
-        }
-        // alternatively every thread takes an equal run of L (column, row) pairs in column-major
-        // order (at most L / rows + 2 column pieces): no ragged last round when N is just above
-        // a multiple of the thread count
-        const long total = (long)N * rows;
-        const long L = (total + nt - 1) / nt;
-        const bool flat = L + 2 * PD * (L / rows + 2) < best;
-        // rows r0 .. r1-1 of column x
-        auto column_run = [&](int x, int r0, int r1) {
-            P a1v[W], a2v[W], w1[W], w2[W];
-#pragma unroll
-            for (int d = 0; d < W; ++d) {
-                a1v[d] = v.pA1[(size_t)x * W + d];
-                a2v[d] = v.pA2 ? v.pA2[(size_t)x * W + d] : P(0);
-                w1[d] = P(0);
-                w2[d] = P(0);
-            }
-            const P* tcol = tbuf + (size_t)r0 * tsp + HO - PD + x;
-            P* rcol = rowbuf + (size_t)r0 * sp + x;
-            for (int r = r0; r < r1 + 2 * PD; ++r) {
-                P t1 = 0, t2 = 0;
-#pragma unroll
-                for (int dk = 0; dk < W; ++dk) {
-                    const P val = tcol[dk];
-                    t1 += a1v[dk] * val;
-                    t2 += a2v[dk] * val;
-                }
-                tcol += tsp;
-#pragma unroll
-                for (int d = 0; d + 1 < W; ++d) {
-                    w1[d] = w1[d + 1];
-                    w2[d] = w2[d + 1];
-                }
-                w1[W - 1] = t1;
-                w2[W - 1] = t2;
-                if (r >= r0 + 2 * PD) {
-                    const P* bj = bco + (size_t)(r - 2 * PD) * 2 * W;
-                    P acc = a.preFscale * *rcol;
-#pragma unroll
-                    for (int dl = 0; dl < W; ++dl) acc = fma(bj[dl], w1[dl], fma(bj[W + dl], w2[dl], acc));
-                    *rcol = acc;
-                    rcol += sp;
-                }
-            }
-        };
-        if (flat) {
-            long s0 = (long)tid * L;
-            const long s1 = min(total, s0 + L);
-            while (s0 < s1) {
-                const int x = (int)(s0 / rows), r0 = (int)(s0 - (long)x * rows);
-                const int r1 = (int)min((long)rows, (long)r0 + (s1 - s0));
-                column_run(x, r0, r1);
-                s0 += r1 - r0;
-            }
-        } else {
-            for (int item = tid; item < N * nh; item += nt) {
-                const int grp = item / N, x = item - grp * N;
-                column_run(x, grp * rh, min(rows, grp * rh + rh));
-            }
-        }
-        __syncthreads();
-    }
-
     // lanes per line: 32 >> (5 - lsh); line r of the CTA = warp * lines-per-warp + lane / lanes
     const int k = lane & ((1 << a.lsh) - 1);
     const int r = (warp << (5 - a.lsh)) + (lane >> a.lsh);
@@ -527,7 +400,6 @@ __global__ void __launch_bounds__(1024) k_ysolve_long(const FastArgs<P> a) {
 
 template <typename P, int PD, bool X>
 cudaError_t run_fast(const LineArgs& a, cudaStream_t s) {
-    constexpr int W = 2 * PD + 1;
     const Chunks& ch = a.f[0].ch;
     if (ch.C > 32) return cudaErrorNotSupported;
     const int mmax = ch.base + 2 * PD;
@@ -553,21 +425,9 @@ cudaError_t run_fast(const LineArgs& a, cudaStream_t s) {
     f.tmax = (P)a.tmax;
     f.b = a.b;
     f.mpad = (ch.base > ch.last ? ch.base : ch.last) | 1;
-    f.preT = (const P*)a.preT;
-    f.preF = (const P*)a.preF;
-    f.preFscale = (P)a.preFscale;
-    f.pc1 = (P)a.pc1;
-    f.pc2 = (P)a.pc2;
-    f.pA1 = (const P*)a.pA1;
-    f.pB1 = (const P*)a.pB1;
-    f.pA2 = (const P*)a.pA2;
-    f.pB2 = (const P*)a.pB2;
-    if (!X && a.preT) return cudaErrorNotSupported;
     if (X) {
         // rows per CTA: as many warps as fit 100 KB of staged rows (at least one)
         const size_t row_bytes = (size_t)a.pitch * sizeof(P);
-        const bool pre = a.preT != nullptr;
-        if (pre && a.narr != 1) return cudaErrorNotSupported;
         // lines per warp: as many as the chunks allow (C <= 8: four, C <= 16: two), or fewer
         int lsh = ch.C <= 8 ? 3 : (ch.C <= 16 ? 4 : 5);
         if (a.rpw == 1) lsh = 5;
@@ -581,11 +441,7 @@ cudaError_t run_fast(const LineArgs& a, cudaStream_t s) {
         if (L < slots)
             while (sp % (2 * L) != L || (sp * sizeof(P)) % 16 != 0) ++sp;
         const size_t srow = (size_t)sp * sizeof(P);
-        const int tsp = pre ? round4(4 + a.pitch + PD) : 0;  // staged T* rows: 4 left, PD right halo
-        const size_t trow = (size_t)tsp * sizeof(P);
-        auto need = [&](int g) {
-            return 128 + g * srow + (pre ? (g + 2 * PD) * trow + (size_t)g * 2 * W * sizeof(P) : 0) + fbytes;
-        };
+        auto need = [&](int g) { return 128 + g * srow + fbytes; };
         // lines per CTA: up to 8 warps' worth, fewer when the staged rows need more than 100 KB
         int G = 8 * lpw;
         if (a.G > 0 && a.G < G) G = a.G < lpw ? lpw : a.G;
@@ -595,14 +451,12 @@ cudaError_t run_fast(const LineArgs& a, cudaStream_t s) {
         if (smem > 227 * 1024) return cudaErrorNotSupported;
         bool aligned = (row_bytes % 16 == 0) && (a.b.sbytes % 16 == 0);
         for (int q = 0; q < a.narr; ++q)
-            aligned = aligned && ((uintptr_t)(pre ? a.preF : a.in[q]) % 16 == 0) && ((uintptr_t)a.out[q] % 16 == 0);
-        if (pre) aligned = aligned && ((uintptr_t)a.preT % 16 == 0);
+            aligned = aligned && ((uintptr_t)a.in[q] % 16 == 0) && ((uintptr_t)a.out[q] % 16 == 0);
         f.G = G;
         f.lsh = lsh;
         f.sp = sp;
-        f.tsp = tsp;
         f.tma = aligned ? 1 : 0;
-        auto kern = pre ? k_xsolve_warp<P, PD, true> : k_xsolve_warp<P, PD, false>;
+        auto kern = k_xsolve_warp<P, PD>;
         cudaError_t e = allow_dynamic_smem(kern, (size_t)smem);
         if (e != cudaSuccess) return e;
         dim3 grid((a.nlines + G - 1) / G, a.narr, a.b.S);
@@ -656,147 +510,6 @@ __global__ void k_pad_factors(const P* __restrict__ luc, const P* __restrict__ s
                               int mmax, P* out) {
     const FacSmem<P, PD> fm(out, mmax);
     fill_factors<P, PD>(luc, spkc, Ec, mmax, fm, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-}
-
-// ---- streaming explicit Kronecker matvec ---------------------------------------------
-// R = Fscale F + c1 (A1^x (x) B1^y) T + c2 (A2^x (x) B2^y) T.  A warp owns 32 columns (lane L
-// <-> column X0 - p + L; lanes p .. 31-p are outputs) and RS output rows: it issues every load
-// of its RS + 2p rows of T and RS rows of F first, x-convolves each row with neighbours'
-// values taken by shuffles, and reduces the y bands from registers.  No shared memory, no
-// barriers, every warp independent.  Values outside the domain are zeros, and the operations
-// (and their order) are those of the right-hand side fused into the x pass.
-template <typename P, int PD, int RS>
-__global__ void __launch_bounds__(128) k_matvec_stream(int Nx, int Ny, int pitch, const P* __restrict__ T,
-                                                       const P* __restrict__ F, P* R, const P* __restrict__ A1,
-                                                       const P* __restrict__ B1, const P* __restrict__ A2,
-                                                       const P* __restrict__ B2, P Fscale, P c1, P c2, Batch b,
-                                                       int nstrips, int nsegs) {
-    constexpr int W = 2 * PD + 1, NR = RS + 2 * PD;
-    if (!scene_active(b)) return;
-    const int lane = threadIdx.x & 31;
-    const int item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (item >= nstrips * nsegs) return;  // whole warp
-    T = scene_ptr(T, b);
-    F = scene_ptr(F, b);
-    R = scene_ptr(R, b);
-    A1 = scene_ptr(A1, b);
-    B1 = scene_ptr(B1, b);
-    A2 = scene_ptr(A2, b);
-    B2 = scene_ptr(B2, b);
-    const int sg = item / nstrips, st = item - sg * nstrips;
-    const int x = st * (32 - 2 * PD) - PD + lane;  // this lane's column
-    const bool xok = x >= 0 && x < Nx;
-    const bool out = lane >= PD && lane < 32 - PD && x < Nx;
-    const int j0 = sg * RS;  // first output row
-    // interior segment: every T row it reads exists and every output row has the interior
-    // y bands (rows 2p .. Ny-2p-1 of a band all equal row 2p), so no row needs a guard
-    const bool yint = j0 >= 2 * PD && j0 + RS + 2 * PD <= Ny;
-    P tv[NR], fv[RS];
-    if (yint) {
-        const P* tp = T + (size_t)(j0 - PD) * pitch + (xok ? x : 0);
-        const P* fp = F + (size_t)j0 * pitch + (xok ? x : 0);
-#pragma unroll
-        for (int i = 0; i < NR; ++i) tv[i] = xok ? tp[(size_t)i * pitch] : P(0);
-#pragma unroll
-        for (int i = 0; i < RS; ++i) fv[i] = out ? fp[(size_t)i * pitch] : P(0);
-    } else {
-#pragma unroll
-        for (int i = 0; i < NR; ++i) {
-            const int r = j0 - PD + i;
-            tv[i] = (xok && r >= 0 && r < Ny) ? T[(size_t)r * pitch + x] : P(0);
-        }
-#pragma unroll
-        for (int i = 0; i < RS; ++i) {
-            const int r = j0 + i;
-            fv[i] = (out && r < Ny) ? F[(size_t)r * pitch + x] : P(0);
-        }
-    }
-    P a1v[W], a2v[W];
-#pragma unroll
-    for (int d = 0; d < W; ++d) {
-        a1v[d] = out ? A1[(size_t)x * W + d] : P(0);
-        a2v[d] = (out && A2) ? A2[(size_t)x * W + d] : P(0);
-    }
-    // x-convolution of every row (outputs lanes read lanes lane - p .. lane + p)
-    P w1[NR], w2[NR];
-    if constexpr (sizeof(P) == 4 && NR % 2 == 0) {
-        // FP32: rows i and i+1 side by side in packed FMAs (per row the same operations)
-        float2 a1p[W], a2p[W];
-#pragma unroll
-        for (int d = 0; d < W; ++d) {
-            a1p[d] = make_float2(a1v[d], a1v[d]);
-            a2p[d] = make_float2(a2v[d], a2v[d]);
-        }
-#pragma unroll
-        for (int i = 0; i < NR; i += 2) {
-            float2 t1 = make_float2(0.f, 0.f), t2 = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int dk = 0; dk < W; ++dk) {
-                const int src = (lane - PD + dk) & 31;
-                const float2 val = (dk == PD) ? make_float2(tv[i], tv[i + 1])
-                                              : make_float2(__shfl_sync(0xffffffffu, tv[i], src),
-                                                            __shfl_sync(0xffffffffu, tv[i + 1], src));
-                t1 = __ffma2_rn(a1p[dk], val, t1);
-                t2 = __ffma2_rn(a2p[dk], val, t2);
-            }
-            w1[i] = t1.x;
-            w1[i + 1] = t1.y;
-            w2[i] = t2.x;
-            w2[i + 1] = t2.y;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < NR; ++i) {
-            P t1 = 0, t2 = 0;
-#pragma unroll
-            for (int dk = 0; dk < W; ++dk) {
-                const P val = (dk == PD) ? tv[i] : __shfl_sync(0xffffffffu, tv[i], (lane - PD + dk) & 31);
-                t1 += a1v[dk] * val;
-                t2 += a2v[dk] * val;
-            }
-            w1[i] = t1;
-            w2[i] = t2;
-        }
-    }
-    if (!out) return;
-    // the interior y bands (rows 2p .. Ny-2p-1 of a band all equal row 2p), where such rows exist
-    const bool has_int = Ny > 4 * PD;
-    P b1i[W], b2i[W];
-#pragma unroll
-    for (int d = 0; d < W; ++d) {
-        b1i[d] = has_int ? c1 * B1[(size_t)(2 * PD) * W + d] : P(0);
-        b2i[d] = (has_int && A2) ? c2 * B2[(size_t)(2 * PD) * W + d] : P(0);
-    }
-    if (yint) {
-        P* rp = R + (size_t)j0 * pitch + x;
-#pragma unroll
-        for (int o = 0; o < RS; ++o) {
-            P acc = Fscale * fv[o];
-#pragma unroll
-            for (int dl = 0; dl < W; ++dl) acc = fma(b1i[dl], w1[o + dl], fma(b2i[dl], w2[o + dl], acc));
-            rp[(size_t)o * pitch] = acc;
-        }
-        return;
-    }
-#pragma unroll
-    for (int o = 0; o < RS; ++o) {
-        const int j = j0 + o;
-        if (j >= Ny) break;
-        P acc = Fscale * fv[o];
-        if (j < 2 * PD || j >= Ny - 2 * PD) {
-            // the first and last 2p rows have bands of their own
-#pragma unroll
-            for (int dl = 0; dl < W; ++dl) {
-                const P b1 = c1 * B1[(size_t)j * W + dl];
-                const P b2 = A2 ? c2 * B2[(size_t)j * W + dl] : P(0);
-                acc = fma(b1, w1[o + dl], fma(b2, w2[o + dl], acc));
-            }
-        } else {
-#pragma unroll
-            for (int dl = 0; dl < W; ++dl) acc = fma(b1i[dl], w1[o + dl], fma(b2i[dl], w2[o + dl], acc));
-        }
-        R[(size_t)j * pitch + x] = acc;
-    }
 }
 
 }  // namespace
@@ -855,37 +568,6 @@ cudaError_t launch_pad_factors(int prec, int p, int mmax, const void* luc, const
         }
     }
 #undef WF_PAD
-    return cudaGetLastError();
-}
-
-cudaError_t launch_matvec(int prec, int p, const MatvecArgs& a, cudaStream_t s) {
-    // output rows per warp item: 16 (the 2p halo rows and the item's setup spread over more
-    // outputs), except 8 for FP64 with p <= 2, where 16 rows would take twice the registers
-    constexpr int WARPS = 4;
-    if (p < 1 || p > 3) return cudaErrorInvalidValue;
-    const int rs = (prec != 0 && p <= 2) ? 8 : 16;
-    const int nstrips = (a.Nx + (32 - 2 * p) - 1) / (32 - 2 * p), nsegs = (a.Ny + rs - 1) / rs;
-    const long items = (long)nstrips * nsegs;
-    dim3 grid((unsigned)((items + WARPS - 1) / WARPS), 1, a.b.S), block(32 * WARPS);
-#define WF_MV(P, PD)                                                                                          \
-    k_matvec_stream<P, PD, (sizeof(P) == 8 && PD <= 2 ? 8 : 16)><<<grid, block, 0, s>>>(                                         \
-        a.Nx, a.Ny, a.pitch, (const P*)a.T, (const P*)a.F, (P*)a.R, (const P*)a.A1, (const P*)a.B1,           \
-        (const P*)a.A2, (const P*)a.B2, (P)a.Fscale, (P)a.c1, (P)a.c2, a.b, nstrips, nsegs)
-    if (prec == 0) {
-        switch (p) {
-            case 1: WF_MV(float, 1); break;
-            case 2: WF_MV(float, 2); break;
-            case 3: WF_MV(float, 3); break;
-        }
-    } else {
-        switch (p) {
-            case 1: WF_MV(double, 1); break;
-            case 2: WF_MV(double, 2); break;
-            case 3: WF_MV(double, 3); break;
-        }
-    }
-#undef WF_MV
-    count_launches(1);
     return cudaGetLastError();
 }
 

@@ -1,34 +1,25 @@
 // Persistent line passes: after the quadrature launch of a Peaceman-Rachford step (one F per
 // step), one launch runs the rest of the step for every active slot of a batch handle.
 //
-// Paper: Sec. 3.1 Eq. matrixPR (the two substeps), Sec. 4 (every directional solve is a set
-// of independent 1-D line solves, which is what lets one launch cover every pass of a whole
-// batch).
+// Paper: Sec. 3.1 Eq. matrixPR (the two substeps, in their combined form, wf_api.cu), Sec. 4
+// (every directional solve is a set of independent 1-D line solves, which is what lets one launch
+// cover every pass of a whole batch).
 //
-// After the quadrature (F, Phi and the substep-1 right-hand side R of every slot), the step of
-// one slot is five passes, each a set of independent tiles:
-//   X1  x lines of R with X_+ and of Phi with M^x, in groups of rows
-//   Y1  y lines (R -> T*, Phi -> phi^{n+1}, increment bases added), in groups of columns
-//   MV  substep-2 right-hand side R = theta F + (A_x (x) M^y) T* + (M^x (x) A_y) T*, eight warp
-//       tiles per item
-//   X2  x lines of R with M^x, in groups of rows
-//   Y2  y lines with Y_+ (R -> T^{n+1}, base T*), guard, in groups of columns
+// After the quadrature (R and Phi of every slot), the step of one slot is two passes, each a set
+// of independent tiles:
+//   X  x lines of R with X_+ and of Phi with M^x, in groups of rows
+//   Y  y lines (R -> T^{n+1} with Y_+, Phi -> phi^{n+1} with M^y, increment bases added, guard),
+//      in groups of columns
 // The arithmetic of every tile is that of the per-pass kernels (the same device functions or
 // the same operations in the same order), so both step forms give the same bits.
 //
-// Work items (pass, slot, tile) are listed by the host in a wavefront over groups of slots: at
-// "time" t the list holds X1 of group t, Y1 of group t-1, ..., Y2 of group t-4, so the fields of
-// about five groups are live at once (sized to stay in the L2 cache: a slot's intermediate
-// fields go from one pass to the next through L2, not HBM), and consecutive items are
-// independent.  A CTA claims the next item from a ticket counter (the next ticket is fetched
-// while the current item runs) and, before touching its inputs, waits for the arrival counters
-// of the tiles it reads:
-//   Y1 columns  <- every X1 row group of its array
-//   MV strip    <- the Y1 column groups that cover its columns and halo
-//   X2 rows     <- the MV segments that cover them (every strip)
-//   Y2 columns  <- every X2 row group
-// A tile waits only for tiles with smaller tickets, which are running or done when it is
-// claimed, so the launch always makes progress whatever the number of resident CTAs.
+// Work items (pass, slot, tiles) are listed by the host in a wavefront over groups of slots: at
+// "time" t the list holds X of group t and Y of group t-1, so the fields of about two groups are
+// live at once, and consecutive items are independent.  A CTA claims the next item from a ticket
+// counter (the next ticket is fetched while the current item runs); before touching its inputs a
+// Y item waits for the arrival counter of the X row groups of its array.  A tile waits only for
+// tiles with smaller tickets, which are running or done when it is claimed, so the launch always
+// makes progress whatever the number of resident CTAs.
 // Producers release (stores, barrier, fence, counter add); consumers acquire (ld.acquire on
 // the counter, barrier) and read data produced in this launch through L2 (ld.global.cg),
 // never through the read-only path.  Every wait is bounded by the handle's wait limit (the
@@ -47,26 +38,18 @@ namespace {
 
 constexpr int kPT = 256;  // threads per CTA
 
-enum { PH_X1 = 0, PH_Y1 = 1, PH_MV = 2, PH_X2 = 3, PH_Y2 = 4, PH_N = 5 };
+enum { PH_X = 0, PH_Y = 1, PH_N = 2 };
 
 // Offsets (ints) of one slot's arrival counters.
 struct CntLayout {
-    int x1, y1col, mvseg, x2, done, stride;
+    int x, done, stride;  // x: one counter per array
 };
 
 template <typename P>
 struct PersistArgs {
-    FastArgs<P> x1, y1, x2, y2;
-    // substep-2 right-hand side
-    const P* mT;
-    const P* mF;
-    P* mR;
-    const P *mA1, *mB1, *mA2, *mB2;
-    P mFscale, mc1, mc2;
-    int mv_nstrips, mv_nsegs;
+    FastArgs<P> x, y;
     long long sbytes;
-    int Nx, Ny, pitch;
-    int nxg, nyg;  // row groups of the x passes, column groups of the y passes
+    int nxg, nyg;  // row groups of the x pass, column groups of the y pass
     int vec;       // rows 16-byte aligned: stage x lines with 16-byte loads
     const int4* items;
     const int* nitems;
@@ -100,7 +83,6 @@ __device__ __forceinline__ LineView<P> line_at(const FastArgs<P>& a, int arr, lo
     v.fpad = nullptr;
     v.status = shift(a.status, off);
     v.tstatus = nullptr;
-    v.preT = v.preF = v.pA1 = v.pB1 = v.pA2 = v.pB2 = nullptr;
     return v;
 }
 
@@ -146,7 +128,7 @@ __device__ __forceinline__ void arrive(int* c) {
 }
 
 // ---- x-line tile (whole CTA): G lines of one array -----------------------------------------
-// The operations of k_xsolve_warp (without the fused right-hand side); rows are staged from L2
+// The operations of k_xsolve_warp; rows are staged from L2
 // with plain loads (they were written by other CTAs of this launch).  `restage`: the factors in
 // shared memory are not those of this (slot, operator).
 template <typename P, int PD>
@@ -303,105 +285,6 @@ __device__ void y_tile(const PersistArgs<P>& A, const FastArgs<P>& a, int z, int
     if (bad && v.status != nullptr && arr == 0) atomicOr(v.status, WF_STATUS_UNSTABLE);
 }
 
-// ---- substep-2 right-hand side tile (one warp): the operations of k_matvec_stream ------------
-template <typename P, int PD, int RS>
-__device__ void mv_tile(const PersistArgs<P>& A, int z, int item) {
-    constexpr int W = 2 * PD + 1, NR = RS + 2 * PD;
-    const int lane = threadIdx.x & 31;
-    const long long off = (long long)z * A.sbytes;
-    const int Nx = A.Nx, Ny = A.Ny;
-    const size_t pitch = (size_t)A.pitch;
-    const P* T = shift(A.mT, off);
-    const P* F = shift(A.mF, off);
-    P* R = shift(A.mR, off);
-    const P* A1 = shift(A.mA1, off);
-    const P* B1 = shift(A.mB1, off);
-    const P* A2 = shift(A.mA2, off);
-    const P* B2 = shift(A.mB2, off);
-    const P Fscale = A.mFscale, c1 = A.mc1, c2 = A.mc2;
-    const int sg = item / A.mv_nstrips, st = item - sg * A.mv_nstrips;
-    const int x = st * (32 - 2 * PD) - PD + lane;
-    const bool xok = x >= 0 && x < Nx;
-    const bool out = lane >= PD && lane < 32 - PD && x < Nx;
-    const int j0 = sg * RS;
-    const bool yint = j0 >= 2 * PD && j0 + RS + 2 * PD <= Ny;
-    P tv[NR], fv[RS];
-    if (yint) {
-        const P* tp = T + (size_t)(j0 - PD) * pitch + (xok ? x : 0);
-        const P* fp = F + (size_t)j0 * pitch + (xok ? x : 0);
-#pragma unroll
-        for (int i = 0; i < NR; ++i) tv[i] = xok ? __ldcg(tp + (size_t)i * pitch) : P(0);
-#pragma unroll
-        for (int i = 0; i < RS; ++i) fv[i] = out ? __ldcg(fp + (size_t)i * pitch) : P(0);
-    } else {
-#pragma unroll
-        for (int i = 0; i < NR; ++i) {
-            const int r = j0 - PD + i;
-            tv[i] = (xok && r >= 0 && r < Ny) ? __ldcg(T + (size_t)r * pitch + x) : P(0);
-        }
-#pragma unroll
-        for (int i = 0; i < RS; ++i) {
-            const int r = j0 + i;
-            fv[i] = (out && r < Ny) ? __ldcg(F + (size_t)r * pitch + x) : P(0);
-        }
-    }
-    P a1v[W], a2v[W];
-#pragma unroll
-    for (int d = 0; d < W; ++d) {
-        a1v[d] = out ? A1[(size_t)x * W + d] : P(0);
-        a2v[d] = (out && A2) ? A2[(size_t)x * W + d] : P(0);
-    }
-    P w1[NR], w2[NR];
-#pragma unroll
-    for (int i = 0; i < NR; ++i) {
-        P t1 = 0, t2 = 0;
-#pragma unroll
-        for (int dk = 0; dk < W; ++dk) {
-            const P val = (dk == PD) ? tv[i] : __shfl_sync(0xffffffffu, tv[i], (lane - PD + dk) & 31);
-            t1 += a1v[dk] * val;
-            t2 += a2v[dk] * val;
-        }
-        w1[i] = t1;
-        w2[i] = t2;
-    }
-    if (!out) return;
-    if (yint) {
-        P b1i[W], b2i[W];
-#pragma unroll
-        for (int d = 0; d < W; ++d) {
-            b1i[d] = c1 * B1[(size_t)(2 * PD) * W + d];
-            b2i[d] = A2 ? c2 * B2[(size_t)(2 * PD) * W + d] : P(0);
-        }
-        P* rp = R + (size_t)j0 * pitch + x;
-#pragma unroll
-        for (int o = 0; o < RS; ++o) {
-            P acc = Fscale * fv[o];
-#pragma unroll
-            for (int dl = 0; dl < W; ++dl) acc = fma(b1i[dl], w1[o + dl], fma(b2i[dl], w2[o + dl], acc));
-            rp[(size_t)o * pitch] = acc;
-        }
-        return;
-    }
-#pragma unroll
-    for (int o = 0; o < RS; ++o) {
-        const int j = j0 + o;
-        if (j >= Ny) break;
-        P acc = Fscale * fv[o];
-#pragma unroll
-        for (int dl = 0; dl < W; ++dl) {
-            const P b1 = c1 * B1[(size_t)j * W + dl];
-            const P b2 = A2 ? c2 * B2[(size_t)j * W + dl] : P(0);
-            acc = fma(b1, w1[o + dl], fma(b2, w2[o + dl], acc));
-        }
-        R[(size_t)j * pitch + x] = acc;
-    }
-}
-
-template <int PD>
-struct MvRows {
-    static constexpr int value = PD > 2 ? 16 : 8;
-};
-
 // ---- the kernel ----------------------------------------------------------------------------
 
 // a slot takes part in this step: active and its step budget not spent
@@ -429,10 +312,9 @@ struct LinesOcc {
 
 template <typename P, int PD>
 __global__ void __launch_bounds__(kPT, LinesOcc<P, PD>::value) k_lines_persist(const __grid_constant__ PersistArgs<P> A) {
-    constexpr int RS = MvRows<PD>::value;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_item, s_go, s_key;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x;
     const int n = *A.nitems;
     int next = 0;
     if (tid == 0) {
@@ -452,69 +334,30 @@ __global__ void __launch_bounds__(kPT, LinesOcc<P, PD>::value) k_lines_persist(c
         int* cnt = A.cnt + (size_t)z * A.cl.stride;
         int* slot_status = shift(A.status, (long long)z * A.sbytes);
         if (tid == 0) {
-            // bit 1: the slot takes part in this step; bit 0: go ahead (the inputs of the item's
-            // tiles are ready: Y1 and Y2 wait once here; X2 and MV per tile below)
+            // bit 1: the slot takes part in this step; bit 0: go ahead (the item's inputs are ready)
             const bool live = slot_live(A, z);
             bool ok = live && !ld_relaxed(A.ctl + 1);
-            if (ok && ph == PH_Y1) ok = wait_count(A, cnt + A.cl.x1 + d.z, A.nxg, slot_status);
-            if (ok && ph == PH_Y2) ok = wait_count(A, cnt + A.cl.x2, A.nxg, slot_status);
+            if (ok && ph == PH_Y) ok = wait_count(A, cnt + A.cl.x + d.z, A.nxg, slot_status);
             s_go = (live ? 2 : 0) | (ok ? 1 : 0);
         }
-        const int key = (z << 4) | (ph << 1) | (ph == PH_MV ? 0 : d.z);  // ph <= 4, arr <= 1: bits 0..3
+        const int key = (z << 2) | (ph << 1) | d.z;  // ph <= 1, arr <= 1
         bool restage = s_key != key;  // read before thread 0 updates it below
         __syncthreads();
         const int go = s_go;
         if (go & 1) {
-            if (ph == PH_MV) {
-                // warp tiles d.z + warp + 8k, k < m; each waits for the Y1 column groups that cover
-                // its strip's columns and halo
-                for (int k = 0; k < m; ++k) {
-                    const int w = d.z + warp + 8 * k;
-                    if (w >= A.mv_nstrips * A.mv_nsegs) break;
-                    const int st = w % A.mv_nstrips;
-                    const int xlo = max(0, st * (32 - 2 * PD) - PD), xhi = min(A.Nx - 1, st * (32 - 2 * PD) - PD + 31);
-                    int ok = 1;
-                    if (lane == 0)
-                        for (int gq = xlo / A.y1.G; gq <= xhi / A.y1.G && ok; ++gq)
-                            ok = wait_count(A, cnt + A.cl.y1col + gq, 1, slot_status) ? 1 : 0;
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
-                    __syncwarp();  // orders the other lanes' loads after lane 0's acquire
-                    if (!ok) break;
-                    mv_tile<P, PD, RS>(A, z, w);
-                    __syncwarp();
-                    if (lane == 0) arrive(cnt + A.cl.mvseg + w / A.mv_nstrips);
-                }
-            } else {
-                const int arr = d.z;
-                const bool xd = ph == PH_X1 || ph == PH_X2;
-                const FastArgs<P>& a = ph == PH_X1 ? A.x1 : (ph == PH_X2 ? A.x2 : (ph == PH_Y1 ? A.y1 : A.y2));
-                for (int k = 0; k < m; ++k) {
-                    const int tile = d.w + k;
-                    if (ph == PH_X2) {
-                        // the MV segments that cover this tile's rows (every strip)
-                        if (tid == 0) {
-                            const int j0 = tile * a.G, j1 = min(a.nlines, j0 + a.G) - 1;
-                            bool ok = true;
-                            for (int sgm = j0 / RS; sgm <= j1 / RS && ok; ++sgm)
-                                ok = wait_count(A, cnt + A.cl.mvseg + sgm, A.mv_nstrips, slot_status);
-                            s_go = ok ? 3 : 2;
-                        }
-                        __syncthreads();
-                        if (!(s_go & 1)) break;
-                    }
-                    if (xd) {
-                        x_tile<P, PD>(A, a, z, arr, tile * a.G, smem, restage, tid, kPT);
-                        __syncthreads();
-                        if (tid == 0) arrive(cnt + (ph == PH_X1 ? A.cl.x1 + arr : A.cl.x2));
-                    } else {
-                        y_tile<P, PD, 16>(A, a, z, arr, tile, smem, restage, tid, kPT);
-                        __syncthreads();
-                        if (tid == 0 && ph == PH_Y1 && arr == 0) arrive(cnt + A.cl.y1col + tile);
-                    }
-                    restage = false;  // the next tile of the item uses the same factors
-                }
-                if (tid == 0) s_key = key;
+            const int arr = d.z;
+            const FastArgs<P>& a = ph == PH_X ? A.x : A.y;
+            for (int k = 0; k < m; ++k) {
+                const int tile = d.w + k;
+                if (ph == PH_X)
+                    x_tile<P, PD>(A, a, z, arr, tile * a.G, smem, restage, tid, kPT);
+                else
+                    y_tile<P, PD, 16>(A, a, z, arr, tile, smem, restage, tid, kPT);
+                __syncthreads();
+                if (tid == 0 && ph == PH_X) arrive(cnt + A.cl.x + arr);
+                restage = false;  // the next tile of the item uses the same factors
             }
+            if (tid == 0) s_key = key;
         }
         if (tid == 0 && (go & 2)) slot_done(A, cnt, z);
         __syncthreads();  // s_item, s_key and the shared memory are reused by the next item
@@ -594,43 +437,22 @@ template <typename P, int PD>
 cudaError_t persist_typed(const PersistHost& h, PersistPlan* plan, bool launch, cudaStream_t s) {
     PersistArgs<P> A;
     memset(&A, 0, sizeof(A));
-    size_t sx1 = 0, sy1 = 0, sx2 = 0, sy2 = 0;
-    if (!fill_line<P, PD>(h.x1, true, h.xG, A.x1, &sx1) || !fill_line<P, PD>(h.y1, false, h.yG, A.y1, &sy1) ||
-        !fill_line<P, PD>(h.x2, true, h.xG, A.x2, &sx2) || !fill_line<P, PD>(h.y2, false, h.yG, A.y2, &sy2))
+    size_t sx = 0, sy = 0;
+    if (!fill_line<P, PD>(h.x, true, h.xG, A.x, &sx) || !fill_line<P, PD>(h.y, false, h.yG, A.y, &sy))
         return cudaErrorNotSupported;
-    if (A.y1.G != A.y2.G || A.x1.G != A.x2.G) return cudaErrorNotSupported;
-    constexpr int RS = MvRows<PD>::value;
-    A.mT = (const P*)h.mv.T;
-    A.mF = (const P*)h.mv.F;
-    A.mR = (P*)h.mv.R;
-    A.mA1 = (const P*)h.mv.A1;
-    A.mB1 = (const P*)h.mv.B1;
-    A.mA2 = (const P*)h.mv.A2;
-    A.mB2 = (const P*)h.mv.B2;
-    A.mFscale = (P)h.mv.Fscale;
-    A.mc1 = (P)h.mv.c1;
-    A.mc2 = (P)h.mv.c2;
-    A.mv_nstrips = (h.mv.Nx + (32 - 2 * PD) - 1) / (32 - 2 * PD);
-    A.mv_nsegs = (h.mv.Ny + RS - 1) / RS;
-    A.sbytes = h.mv.b.sbytes;
-    A.Nx = h.mv.Nx;
-    A.Ny = h.mv.Ny;
-    A.pitch = h.mv.pitch;
-    A.nxg = (h.x1.nlines + A.x1.G - 1) / A.x1.G;
-    A.nyg = (h.y1.nlines + A.y1.G - 1) / A.y1.G;
-    bool vec = sizeof(P) == 4 && (h.mv.pitch % 4) == 0 && (A.sbytes % 16) == 0;
-    for (const LineArgs* la : {&h.x1, &h.x2})
-        for (int q = 0; q < la->narr; ++q) vec = vec && ((uintptr_t)la->in[q] % 16 == 0) && ((uintptr_t)la->out[q] % 16 == 0);
+    A.sbytes = h.x.b.sbytes;
+    A.nxg = (h.x.nlines + A.x.G - 1) / A.x.G;
+    A.nyg = (h.y.nlines + A.y.G - 1) / A.y.G;
+    bool vec = sizeof(P) == 4 && (h.x.pitch % 4) == 0 && (A.sbytes % 16) == 0;
+    for (int q = 0; q < h.x.narr; ++q)
+        vec = vec && ((uintptr_t)h.x.in[q] % 16 == 0) && ((uintptr_t)h.x.out[q] % 16 == 0);
     A.vec = vec ? 1 : 0;
     CntLayout cl;
-    cl.x1 = 0;
-    cl.y1col = cl.x1 + 2;
-    cl.mvseg = cl.y1col + A.nyg;
-    cl.x2 = cl.mvseg + A.mv_nsegs;
-    cl.done = cl.x2 + 1;
-    cl.stride = (cl.done + 1 + 31) & ~31;  // 128-byte blocks per slot
+    cl.x = 0;
+    cl.done = 2;
+    cl.stride = 32;  // a 128-byte block per slot
     A.cl = cl;
-    const size_t smem = std::max(std::max(sx1, sx2), std::max(sy1, sy2));
+    const size_t smem = std::max(sx, sy);
     auto kern = k_lines_persist<P, PD>;
     cudaError_t e = allow_dynamic_smem(kern, (size_t)smem);
     if (e != cudaSuccess) return e;
@@ -638,17 +460,11 @@ cudaError_t persist_typed(const PersistHost& h, PersistPlan* plan, bool launch, 
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPT, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorNotSupported;
-    plan->nq = 0;
-    plan->nmv = A.mv_nstrips * A.mv_nsegs;  // warp tiles
     plan->nxg = A.nxg;
     plan->nyg = A.nyg;
-    plan->narr1 = h.x1.narr;
+    plan->narr = h.x.narr;
     plan->cstride = cl.stride;
     plan->ctas = per_sm * sm_count();
-    plan->seg = 0;
-    plan->xG = A.x1.G;
-    plan->yG = A.y1.G;
-    plan->smem = smem;
     if (!launch) return cudaSuccess;
     // the item list and counters were laid out for this plan (prepare step): never write past them
     if (!h.items || !h.ctl || !h.cnt || (size_t)h.nslots_cap * cl.stride > h.cnt_cap) return cudaErrorInvalidValue;
@@ -712,10 +528,8 @@ int persist_items(const PersistPlan& plan, const int* slots, int nslots, int gs,
     auto per_item = [&](long tiles_all, int most) {
         return (int)std::max(1L, std::min((long)most, tiles_all / target));
     };
-    const int tx = per_item((long)nslots * plan.narr1 * plan.nxg, plan.nxg);
-    const int ty = per_item((long)nslots * plan.narr1 * plan.nyg, plan.nyg);
-    const int mv8 = (plan.nmv + 7) / 8;  // CTA rounds of eight warp tiles
-    const int tm = per_item((long)nslots * mv8, mv8);
+    const int tx = per_item((long)nslots * plan.narr * plan.nxg, plan.nxg);
+    const int ty = per_item((long)nslots * plan.narr * plan.nyg, plan.nyg);
     int n = 0, per_slot = 0;
     auto put = [&](int ph, int m, int z, int a, int b) {
         if (n < cap) out[n] = make_int4(ph | (m << 8), z, a, b);
@@ -731,23 +545,8 @@ int persist_items(const PersistPlan& plan, const int* slots, int nslots, int gs,
             for (int k = g * gs; k < std::min(nslots, (g + 1) * gs); ++k) {
                 const int z = slots[k];
                 const int n0 = n;
-                switch (ph) {
-                    case PH_X1:
-                        for (int arr = 0; arr < plan.narr1; ++arr) tiles(PH_X1, z, arr, plan.nxg, tx);
-                        break;
-                    case PH_Y1:
-                        for (int arr = 0; arr < plan.narr1; ++arr) tiles(PH_Y1, z, arr, plan.nyg, ty);
-                        break;
-                    case PH_MV:
-                        for (int i = 0; i < mv8; i += tm) put(PH_MV, std::min(tm, mv8 - i), z, 8 * i, 0);
-                        break;
-                    case PH_X2:
-                        tiles(PH_X2, z, 0, plan.nxg, tx);
-                        break;
-                    case PH_Y2:
-                        tiles(PH_Y2, z, 0, plan.nyg, ty);
-                        break;
-                }
+                for (int arr = 0; arr < plan.narr; ++arr)
+                    tiles(ph, z, arr, ph == PH_X ? plan.nxg : plan.nyg, ph == PH_X ? tx : ty);
                 if (k == 0) per_slot += n - n0;
             }
         }
