@@ -62,10 +62,8 @@ struct Dir {
     int n = 0, N = 0;
     double L = 0, h = 0;
     Chunks ch{};
-    ElemTabs itab{};  // host copy of the interior element's tables
     // shared by all slots
     double *B64 = nullptr, *D64 = nullptr;
-    void *BP = nullptr, *DP = nullptr, *wP = nullptr;
     double *M64 = nullptr, *K64 = nullptr, *G64 = nullptr;
     // per slot
     Op op[3];  // 0: M, 1: -theta A (explicit side, band only), 2: M + theta A (implicit side)
@@ -144,6 +142,7 @@ struct wf_handle {
     bool noalloc_run = false;  // wf_step_noalloc in progress: per-pass launches only
     void *T = nullptr, *phi = nullptr, *Phi = nullptr, *R = nullptr;
     int* status = nullptr;
+    void* mw = nullptr;  // mean wind (2 values)
     void *fxq = nullptr, *gxq = nullptr, *fyq = nullptr, *gyq = nullptr;
     std::vector<Slot> slots;
     std::vector<int> active_host;
@@ -164,6 +163,16 @@ struct wf_handle {
 namespace wf {
 std::atomic<unsigned long long> g_launches{0};
 void count_launches(int n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
+
+cudaError_t launch_rhs(int prec, int p, const RhsArgs& a, cudaStream_t s) {
+    const bool f32 = prec == WF_FP32;
+    switch (p) {
+        case 1: return f32 ? launch_quad_p1_f32(a, s) : launch_quad_p1_f64(a, s);
+        case 2: return f32 ? launch_quad_p2_f32(a, s) : launch_quad_p2_f64(a, s);
+        case 3: return f32 ? launch_quad_p3_f32(a, s) : launch_quad_p3_f64(a, s);
+    }
+    return cudaErrorInvalidValue;
+}
 }  // namespace wf
 
 namespace {
@@ -230,15 +239,6 @@ void layout_shared(wf_handle* h, Arena& A) {
         const size_t tab = (size_t)d->n * h->q * (h->p + 1);
         d->B64 = A.take<double>(tab);
         d->D64 = A.take<double>(tab);
-        if (h->prec == WF_FP32) {
-            d->BP = A.take<float>(tab);
-            d->DP = A.take<float>(tab);
-            d->wP = A.take<float>(16);
-        } else {
-            d->BP = d->B64;
-            d->DP = d->D64;
-            d->wP = A.take<double>(16);
-        }
         d->M64 = A.take<double>((size_t)d->N * W);
         d->K64 = A.take<double>((size_t)d->N * W);
         d->G64 = A.take<double>((size_t)d->N * W);
@@ -288,6 +288,7 @@ void layout_slot(wf_handle* h, Arena& A) {
         }
     }
     const size_t qx = (size_t)kMaxRank * h->nx * h->q, qy = (size_t)kMaxRank * h->ny * h->q;
+    h->mw = A.take<char>(2 * es);
     h->fxq = A.take<char>(qx * es);
     h->gxq = A.take<char>(qy * es);
     h->fyq = A.take<char>(qx * es);
@@ -355,51 +356,6 @@ int build_tables(wf_handle* h) {
     for (Dir* d : ds) {
         WF_TRY(launch_basis(h->gxi, h->q, d->n, h->p, d->L, d->B64, d->D64, s));
         WF_TRY(launch_assemble(d->B64, d->D64, h->gw, h->q, d->n, h->p, d->h, d->M64, d->K64, d->G64, s));
-        const size_t tab = (size_t)d->n * h->q * (h->p + 1);
-        if (h->prec == WF_FP32) {
-            WF_TRY(launch_to_f32(d->B64, (float*)d->BP, tab, s));
-            WF_TRY(launch_to_f32(d->D64, (float*)d->DP, tab, s));
-        }
-    }
-    double w[16];
-    WF_TRY(cudaMemcpyAsync(w, h->gw, sizeof(double) * h->q, cudaMemcpyDeviceToHost, s));
-    WF_TRY(cudaStreamSynchronize(s));
-    for (Dir* d : ds) {
-        if (h->prec == WF_FP32) {
-            float wf32[16];
-            for (int a = 0; a < h->q; ++a) wf32[a] = (float)(w[a] * d->h);
-            WF_TRY(cudaMemcpyAsync(d->wP, wf32, sizeof(float) * h->q, cudaMemcpyHostToDevice, s));
-        } else {
-            double w64[16];
-            for (int a = 0; a < h->q; ++a) w64[a] = w[a] * d->h;
-            WF_TRY(cudaMemcpyAsync(d->wP, w64, sizeof(double) * h->q, cudaMemcpyHostToDevice, s));
-        }
-        WF_TRY(cudaStreamSynchronize(s));  // the host weight arrays go out of scope
-        // interior element p (uniform knots): its tables, read back once
-        ElemTabs& it = d->itab;
-        memset(&it, 0, sizeof(it));
-        for (int a = 0; a < h->q; ++a) it.w[a] = w[a] * d->h;
-        it.ok = d->n > 2 * h->p;
-        if (it.ok) {
-            const int Q = h->q, NB = h->p + 1;
-            double tb[16], td[16];
-            const size_t off = (size_t)h->p * Q * NB;
-            WF_TRY(cudaMemcpyAsync(tb, d->B64 + off, sizeof(double) * Q * NB, cudaMemcpyDeviceToHost, s));
-            WF_TRY(cudaMemcpyAsync(td, d->D64 + off, sizeof(double) * Q * NB, cudaMemcpyDeviceToHost, s));
-            WF_TRY(cudaStreamSynchronize(s));
-            for (int a = 0; a < Q; ++a)
-                for (int k = 0; k < NB; ++k) {
-                    it.B[a][k] = tb[a * NB + k];
-                    it.D[a][k] = td[a * NB + k];
-                }
-        }
-        // an interior row of the mass matrix (assembled from the same element tables)
-        const int W = 2 * h->p + 1;
-        if (d->N >= 4 * h->p + 1) {
-            WF_TRY(cudaMemcpyAsync(it.Mb, d->M64 + (size_t)(2 * h->p) * W, sizeof(double) * W,
-                                   cudaMemcpyDeviceToHost, s));
-            WF_TRY(cudaStreamSynchronize(s));
-        }
     }
     return WF_OK;
 }
@@ -455,7 +411,16 @@ int build_factors(wf_handle* h, int slot, double tol, double* worst) {
             if (o.factored)
                 WF_TRY(launch_pad_factors(h->prec, h->p, o.mmax, at(h, o.lucP, slot), at(h, o.spkcP, slot),
                                           at(h, o.EcP, slot), at(h, o.fpadP, slot), s));
-    WF_TRY(cudaStreamSynchronize(s));
+    const Slot& sl = h->slots[slot];
+    if (h->prec == WF_FP32) {
+        const float b[2] = {(float)sl.wind_x, (float)sl.wind_y};
+        WF_TRY(cudaMemcpyAsync(at(h, h->mw, slot), b, sizeof(b), cudaMemcpyHostToDevice, s));
+        WF_TRY(cudaStreamSynchronize(s));  // b goes out of scope
+    } else {
+        const double b[2] = {sl.wind_x, sl.wind_y};
+        WF_TRY(cudaMemcpyAsync(at(h, h->mw, slot), b, sizeof(b), cudaMemcpyHostToDevice, s));
+        WF_TRY(cudaStreamSynchronize(s));
+    }
     return *worst > tol ? WF_ETRUNC : WF_OK;
 }
 
@@ -504,48 +469,31 @@ cudaError_t timed(wf_handle* h, int site, F&& launch) {
     return e;
 }
 
-// R = Rscale F + c1 (A1 (x) B1) T + c2 (A2 (x) B2) T  (A2 == nullptr drops the second term)
-RhsArgs rhs_args(wf_handle* h, const void* T, void* F, void* Phi, void* R, double Rscale, const Op& A1,
-                 const Op& B1, double c1, const Op* A2, const Op* B2, double c2) {
+// Quadrature: R = Rscale (F - A_x (x) M^y T - M^x (x) A_y T) (xonly: without the y operator), and Phi
+RhsArgs rhs_args(wf_handle* h, void* Phi, void* R, double Rscale, bool xonly) {
     RhsArgs a;
     a.nx = h->nx;
     a.ny = h->ny;
     a.Nx = h->Nx;
     a.Ny = h->Ny;
     a.pitch = h->pitch;
-    a.T = T;
+    a.hx = h->dx.h;
+    a.hy = h->dy.h;
+    a.T = h->T;
     a.phi = h->phi;
-    a.F = F;
     a.Phi = Phi;
     a.R = R;
-    a.Bx = h->dx.BP;
-    a.Dx = h->dx.DP;
-    a.By = h->dy.BP;
-    a.Dy = h->dy.DP;
-    a.wx = h->dx.wP;
-    a.wy = h->dy.wP;
+    a.xonly = xonly ? 1 : 0;
+    a.Rscale = Rscale;
+    a.tau = h->dt;
     a.wind_rank = h->wr;
     a.fxq = h->fxq;
     a.gxq = h->gxq;
     a.fyq = h->fyq;
     a.gyq = h->gyq;
-    a.A1 = A1.bandP;
-    a.B1 = B1.bandP;
-    a.A2 = A2 ? A2->bandP : nullptr;
-    a.B2 = B2 ? B2->bandP : nullptr;
-    a.Rscale = Rscale;
-    a.c1 = c1;
-    a.c2 = c2;
-    a.tau = h->dt;
+    a.mw = h->mw;
     a.seg = h->tune[2];
-    // the boundary items' stream (both slot groups of step form 3 fork to it in turn: a group's
-    // quadrature joins back before its line passes, and group B's starts after group A's)
-    a.aux = h->aux;
-    a.ev_fork = h->ev_fork;
-    a.ev_join = h->ev_join;
-    a.single = 0;
-    a.tx = h->dx.itab;
-    a.ty = h->dy.itab;
+    a.parts = 0;
     a.phys = h->phys;
     a.b = batch(h);
     return a;
@@ -612,12 +560,11 @@ cudaError_t upload_active(wf_handle* h) {
 //   (X_+ (x) M^y) (T^{n+1} - T**) = tau/2 F(T**) - 2 theta_x (A_x (x) M^y) T**
 // Rounding errors then scale with the increment instead of the temperature,
 // which keeps the FP32 path accurate through the inverse mass matrices.
-// quadrature launch, then (with a manufactured solution) its forcing: out1 += s1 int f B,
-// out2 += s2 int f B
-cudaError_t rhs_and_forcing(wf_handle* h, const RhsArgs& r, void* out1, double s1, void* out2, double s2) {
+// quadrature launch, then (with a manufactured solution) its forcing: R += Rscale int f B
+cudaError_t rhs_and_forcing(wf_handle* h, const RhsArgs& r) {
     cudaError_t e = launch_rhs(h->prec, h->p, r, h->stream);
     if (e != cudaSuccess || !h->mms_on) return e;
-    return launch_forcing(h->prec, h->mms, out1, s1, out2, s2, h->stream);
+    return launch_forcing(h->prec, h->mms, r.R, r.Rscale, h->stream);
 }
 
 cudaError_t enqueue_step_body(wf_handle* h);
@@ -797,8 +744,8 @@ cudaError_t enqueue_step_body(wf_handle* h) {
     cudaError_t e;
     if (h->prm.scheme == WF_EXPLICIT) {
         // (M^x (x) M^y)(T^{n+1} - T^n) = tau F - tau (A_x (x) M^y) T^n - tau (M^x (x) A_y) T^n
-        RhsArgs r1 = rhs_args(h, h->T, nullptr, h->Phi, h->R, h->dt, X[1], Y[0], 1.0, &X[0], &Y[1], 1.0);
-        auto l1 = [&] { return rhs_and_forcing(h, r1, h->R, h->dt, nullptr, 0.0); };
+        RhsArgs r1 = rhs_args(h, h->Phi, h->R, h->dt, false);
+        auto l1 = [&] { return rhs_and_forcing(h, r1); };
         if ((e = timed(h, S_RHS1, l1)) != cudaSuccess) return e;
         if (h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return e;
         LineArgs x1 = line_args(h, 1);
@@ -813,11 +760,12 @@ cudaError_t enqueue_step_body(wf_handle* h) {
         return cudaSuccess;
     }
     if (h->prm.scheme == WF_PR && h->prm.F_timing == WF_F_ONCE) {
-        // R = tau F + 2 (op1_x (x) M^y) T + 2 (M^x (x) op1_y) T, then X_+ lines along x, Y_+ along y
-        RhsArgs r1 = rhs_args(h, h->T, nullptr, h->Phi, h->R, h->dt, X[1], Y[0], 2.0, &X[0], &Y[1], 2.0);
+        // X_+ lines along x, Y_+ along y.  Step form 1: a launch per array and per kind of strip
+        RhsArgs r1 = rhs_args(h, h->Phi, h->R, h->dt, false);
         const bool pers = use_persist(h) && h->p_ctl;
-        r1.single = pers ? 1 : 0;  // the quadrature in one launch: two launches per step in all
-        auto l1 = [&] { return rhs_and_forcing(h, r1, h->R, h->dt, nullptr, 0.0); };
+        const bool split = h->tune[6] == 1 || (h->tune[6] == 3 && h->gn == 0);
+        r1.parts = split ? 1 : 0;
+        auto l1 = [&] { return rhs_and_forcing(h, r1); };
         if ((e = timed(h, S_RHS1, l1)) != cudaSuccess) return e;
         if (h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return e;
         if (pers) {
@@ -825,8 +773,6 @@ cudaError_t enqueue_step_body(wf_handle* h) {
             persist_args(h, &ph);
             return timed(h, S_PERSIST, [&] { return persist_step(ph, nullptr, true, s); });
         }
-        // both arrays in one launch per direction; step form 1: a launch per array
-        const bool split = h->tune[6] == 1 || (h->tune[6] == 3 && h->gn == 0);
         for (int part = 0; part < (split ? 2 : 1); ++part) {
             LineArgs x1 = line_args(h, 1);
             if (part == 0) add_line(x1, h->R, h->R, X[2], cx);
@@ -845,8 +791,8 @@ cudaError_t enqueue_step_body(wf_handle* h) {
     if (h->prm.scheme == WF_PR) {
         // F re-evaluated at T* in the second substep
         const double th = 0.5 * h->dt;
-        RhsArgs r1 = rhs_args(h, h->T, nullptr, h->Phi, h->R, th, X[1], Y[0], 1.0, &X[0], &Y[1], 1.0);
-        auto l1 = [&] { return rhs_and_forcing(h, r1, h->R, th, nullptr, 0.0); };
+        RhsArgs r1 = rhs_args(h, h->Phi, h->R, th, false);
+        auto l1 = [&] { return rhs_and_forcing(h, r1); };
         if ((e = timed(h, S_RHS1, l1)) != cudaSuccess) return e;
         if (h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return e;
         LineArgs x1 = line_args(h, 1);
@@ -856,8 +802,8 @@ cudaError_t enqueue_step_body(wf_handle* h) {
         LineArgs y1 = line_args(h, 0);
         add_line(y1, h->R, h->T, Y[0], cy, h->T);
         if ((e = timed(h, S_Y1, [&] { return launch_ysolve(prec, p, y1, s); })) != cudaSuccess) return e;
-        RhsArgs r2 = rhs_args(h, h->T, nullptr, nullptr, h->R, th, X[1], Y[0], 1.0, &X[0], &Y[1], 1.0);
-        auto l2 = [&] { return rhs_and_forcing(h, r2, h->R, th, nullptr, 0.0); };
+        RhsArgs r2 = rhs_args(h, nullptr, h->R, th, false);
+        auto l2 = [&] { return rhs_and_forcing(h, r2); };
         if ((e = timed(h, S_RHS2, l2)) != cudaSuccess) return e;
         LineArgs x2 = line_args(h, 2);
         add_line(x2, h->R, h->R, X[0], cx);
@@ -871,8 +817,8 @@ cudaError_t enqueue_step_body(wf_handle* h) {
     }
     // Strang / Crank-Nicolson
     const double half = 0.5 * h->dt;
-    RhsArgs r1 = rhs_args(h, h->T, nullptr, h->Phi, h->R, half, X[1], Y[0], 2.0, nullptr, nullptr, 0.0);
-    auto l1 = [&] { return rhs_and_forcing(h, r1, h->R, half, nullptr, 0.0); };
+    RhsArgs r1 = rhs_args(h, h->Phi, h->R, half, true);
+    auto l1 = [&] { return rhs_and_forcing(h, r1); };
     if ((e = timed(h, S_RHS1, l1)) != cudaSuccess) return e;
     if (h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return e;
     LineArgs x1 = line_args(h, 1);
@@ -885,8 +831,8 @@ cudaError_t enqueue_step_body(wf_handle* h) {
     LineArgs yy = line_args(h, 0);
     add_line(yy, h->T, h->T, Y[2], cy, h->T, Y[1].bandP, 2.0);
     if ((e = timed(h, S_Y2PRE, [&] { return launch_ysolve(prec, p, yy, s); })) != cudaSuccess) return e;
-    RhsArgs r2 = rhs_args(h, h->T, nullptr, nullptr, h->R, half, X[1], Y[0], 2.0, nullptr, nullptr, 0.0);
-    auto l2 = [&] { return rhs_and_forcing(h, r2, h->R, half, nullptr, 0.0); };
+    RhsArgs r2 = rhs_args(h, nullptr, h->R, half, true);
+    auto l2 = [&] { return rhs_and_forcing(h, r2); };
     if ((e = timed(h, S_RHS2, l2)) != cudaSuccess) return e;
     LineArgs x2 = line_args(h, 2);
     add_line(x2, h->R, h->R, X[2], cx);

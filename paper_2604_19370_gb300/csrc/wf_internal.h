@@ -1,11 +1,11 @@
 // Internal declarations shared by the CUDA translation units of libwf.
 //
 // Data layout on the device (all fields of one handle):
-//   - coefficient fields T, phi, F, Phi, R: [Ny][pitch] in the handle's
+//   - coefficient fields T, phi, Phi, R: [Ny][pitch] in the handle's
 //     precision P (float or double), pitch = Nx rounded up to 32 elements
 //     so every row starts on a 128-byte boundary;
 //   - 1-D Gauss tables per direction: B[e][a][l] = B_{e+l}(x_{e,a}) and the
-//     derivative D[e][a][l], e < n, a < q = p+1, l <= p; weights w[a]*h;
+//     derivative D[e][a][l], e < n, a < q = p+1, l <= p;
 //   - 1-D banded matrices: band[r][d] = A[r][r+d-p], d in [0, 2p], zero
 //     outside the matrix;
 //   - chunked LU factors of a 1-D operator (see Factor below).
@@ -128,47 +128,34 @@ cudaError_t launch_gather_status(int* status0, long long sbytes, int S, int* out
 // skipped by every kernel until its budget is set again)
 cudaError_t launch_step_budget(const int* active, int* budget, int S, cudaStream_t s);
 
-// ---- quadrature right-hand side (wf_rhs.cu) ---------------------------------------
-// Tables of an interior element along one direction (uniform open knots: every element
-// p <= e < n - p has the same ones, bitwise, as the device tables), and the Gauss weights.
-struct ElemTabs {
-    int ok;                   // n > 2p (interior elements exist)
-    double B[4][4], D[4][4];  // [Gauss point][local basis], as in the device tables
-    double w[4];              // Gauss weight x element length
-    double Mb[8];             // band of an interior row of the 1-D mass matrix (rows 2p .. N-1-2p)
-};
-
+// ---- quadrature (wf_quad.cuh) -------------------------------------------------------
 struct RhsArgs {
     int nx, ny, Nx, Ny, pitch;
+    double hx, hy;  // element sizes
     const void* T;
     const void* phi;
-    void* F;    // temperature load vector (optional)
     void* Phi;  // fuel increment load vector -tau k_f int(E phi B_i B_j) (optional)
-    void* R;    // Rscale F + c1 (A1 (x) B1) T + c2 (A2 (x) B2) T (optional)
-    const void *Bx, *Dx, *By, *Dy, *wx, *wy;
+    void* R;    // Rscale (F - A_x (x) M^y T - M^x (x) A_y T), or with xonly Rscale (F - A_x (x) M^y T)
+    int xonly;
+    double Rscale;
+    double tau;  // full time step (fuel update)
     int wind_rank;
     const void *fxq, *gxq, *fyq, *gyq;  // [rank][n*q] factor values at Gauss points
-    const void *A1, *B1, *A2, *B2;      // bands along x (A) and y (B) for R; A2 may be NULL
-    double Rscale, c1, c2;
-    double tau;  // full time step (fuel update)
-    int seg;     // element rows per segment of the streaming kernel (0: the launcher's rule)
-    // second stream and fork/join events of the handle: the quadrature's boundary items run
-    // there, beside its interior items (NULL: one stream)
-    cudaStream_t aux;
-    cudaEvent_t ev_fork, ev_join;
-    int single;  // FP32: all items in one launch (no second stream)
-    ElemTabs tx, ty;
+    const void* mw;                     // mean wind (b_x, b_y)
+    int seg;    // rows per segment (0: the launcher's rule)
+    int parts;  // FP32: the strips at either x boundary in launches of their own
     Phys phys;
-    Batch b;  // per scenario: T, phi, F, Phi, R, A1, B1, A2, B2, fxq, gxq, fyq, gyq
+    Batch b;  // per scenario: T, phi, Phi, R, mw, fxq, gxq, fyq, gyq
 };
 cudaError_t launch_rhs(int prec, int p, const RhsArgs& a, cudaStream_t s);
+cudaError_t launch_quad_p1_f32(const RhsArgs& a, cudaStream_t s);
+cudaError_t launch_quad_p2_f32(const RhsArgs& a, cudaStream_t s);
+cudaError_t launch_quad_p3_f32(const RhsArgs& a, cudaStream_t s);
+cudaError_t launch_quad_p1_f64(const RhsArgs& a, cudaStream_t s);
+cudaError_t launch_quad_p2_f64(const RhsArgs& a, cudaStream_t s);
+cudaError_t launch_quad_p3_f64(const RhsArgs& a, cudaStream_t s);
 // process-wide count of the time-step kernels launched (wf_launch_count)
 void count_launches(int n);
-// streaming form of the same computation (wf_rhs_stream.cu); cudaErrorNotSupported for
-// a wind variation of rank > 2
-cudaError_t launch_rhs_stream(int prec, int p, const RhsArgs& a, cudaStream_t s);
-cudaError_t launch_rhs_tile(int prec, int p, const RhsArgs& a, cudaStream_t s);  // shared-memory tiles
-int rhs_items_per_dof(int p);  // informational
 
 // ---- manufactured-solution forcing (wf_mms.cu) --------------------------------------
 struct MmsArgs {
@@ -181,9 +168,8 @@ struct MmsArgs {
     double C_d, c_W, c_chi, T_amb, T_amb4, c_rad, C_nld, wind_x, wind_y;
     const double* t;        // device: start time of the step being enqueued
 };
-// out1 += s1 * int f B_i B_j, and out2 += s2 * the same when out2 is not NULL
-cudaError_t launch_forcing(int prec, const MmsArgs& a, void* out1, double s1, void* out2, double s2,
-                           cudaStream_t s);
+// out += s1 * int f B_i B_j
+cudaError_t launch_forcing(int prec, const MmsArgs& a, void* out, double s1, cudaStream_t s);
 cudaError_t launch_advance_time(double* t, double dt, cudaStream_t s);
 
 // ---- line solves (wf_solve.cu) -------------------------------------------

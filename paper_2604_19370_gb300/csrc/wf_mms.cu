@@ -42,7 +42,7 @@ __device__ double mms_forcing(const MmsArgs& a, double x, double y, double t) {
 
 // one thread per DOF (i, j): sum over the (p+1)^2 elements of its support and their q^2 points
 template <typename P>
-__global__ void k_forcing(MmsArgs a, P* out1, P s1, P* out2, P s2) {
+__global__ void k_forcing(MmsArgs a, P* out, P s1) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     if (i >= a.Nx || j >= a.Ny) return;
@@ -67,8 +67,7 @@ __global__ void k_forcing(MmsArgs a, P* out1, P s1, P* out2, P s2) {
         }
     }
     const size_t g = (size_t)j * a.pitch + i;
-    out1[g] += s1 * (P)acc;
-    if (out2) out2[g] += s2 * (P)acc;
+    out[g] += s1 * (P)acc;
 }
 
 __global__ void k_advance_time(double* t, double dt) {
@@ -77,13 +76,12 @@ __global__ void k_advance_time(double* t, double dt) {
 
 }  // namespace
 
-cudaError_t launch_forcing(int prec, const MmsArgs& a, void* out1, double s1, void* out2, double s2,
-                           cudaStream_t s) {
+cudaError_t launch_forcing(int prec, const MmsArgs& a, void* out, double s1, cudaStream_t s) {
     dim3 block(32, 4), grid((a.Nx + 31) / 32, (a.Ny + 3) / 4);
     if (prec == 0)
-        k_forcing<float><<<grid, block, 0, s>>>(a, (float*)out1, (float)s1, (float*)out2, (float)s2);
+        k_forcing<float><<<grid, block, 0, s>>>(a, (float*)out, (float)s1);
     else
-        k_forcing<double><<<grid, block, 0, s>>>(a, (double*)out1, s1, (double*)out2, s2);
+        k_forcing<double><<<grid, block, 0, s>>>(a, (double*)out, s1);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -1,0 +1,8 @@
+// Quadrature kernels of degree 2, FP32 (see wf_quad.cuh).
+#include "wf_quad.cuh"
+
+namespace wf {
+
+cudaError_t launch_quad_p2_f32(const RhsArgs& r, cudaStream_t s) { return quad_by_rank<float, 2>(r, s); }
+
+}  // namespace wf
