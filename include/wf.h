@@ -250,19 +250,14 @@ int wf_launch_count(unsigned long long* n);
 /*
  * Launch-shape autotuner (no counterpart in the paper, whose solver runs on
  * CPU threads).  Eight values are tuned (int shape[8]):
- *   shape[0]  lines per CTA of the first x pass of a step (rows staged per
- *             CTA; at most 8 warps' worth); lines per tile of both x passes of
- *             the persistent step,
- *   shape[1]  lines per CTA of the y pass (columns per CTA, bounded by
- *             lines x chunks <= 256 threads); columns per tile of the
- *             persistent step's y passes,
- *   shape[2]  element rows per segment of the streaming quadrature kernel,
- *   shape[3]  lines per warp of the x passes (1, 2 or 4; at most 32 / chunks
- *             per line, which is also the default),
- *   shape[4]  lines per CTA of the second x pass,
- *   shape[5]  accepted and ignored (it placed the right-hand side of the second
- *             x pass of Peaceman-Rachford with one F per step, whose combined
- *             form has no second x pass);
+ *   shape[0]  rows per CTA of the first x pass of a step (a power of two up to
+ *             8 is used) and of the x tiles of the persistent step,
+ *   shape[2]  rows per segment of the quadrature kernel,
+ *   shape[4]  rows per CTA of the second x pass (Strang / Crank-Nicolson, F per
+ *             substep),
+ *   shape[1], shape[3], shape[5]  accepted and ignored (columns per CTA of the y
+ *             passes, lines per warp and the place of the second right-hand
+ *             side, which have one form now);
  *   shape[6]  step form: 0 one launch per direction (T and fuel side by
  *             side), 1 Peaceman-Rachford with one F per step: one launch per
  *             direction and array (seven per step in FP32; elsewhere as 0),
@@ -486,7 +481,7 @@ void wf_server_destroy(wf_server* s);
  * tables and factors; T and fuel are device arrays of Ny rows with a row pitch of
  * `pitch` >= Nx float elements, updated in place.  The intermediate fields of
  * the step live in one static device array that the library reserves on every
- * GPU it is loaded on (4 MiB, held until the process exits); pitch * Ny must not
+ * GPU it is loaded on (6 MiB, held until the process exits); pitch * Ny must not
  * exceed 524288 (512 x 512 elements of degree 2 fit).  The first call on a
  * device looks up that array's device address; make that first call before any
  * stream capture.  All calls share the array: two calls whose work overlaps on

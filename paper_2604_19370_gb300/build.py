@@ -22,8 +22,9 @@ OUT = os.path.join(HERE, "_build")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(OUT, "libwf.so")
 
-SOURCES = ["wf_tables.cu", "wf_quad_p1_f32.cu", "wf_quad_p2_f32.cu", "wf_quad_p3_f32.cu", "wf_quad_p1_f64.cu", "wf_quad_p2_f64.cu",
-           "wf_quad_p3_f64.cu", "wf_solve.cu", "wf_linefast.cu", "wf_api.cu", "wf_server.cu", "wf_mms.cu", "wf_probe.cu", "wf_persist.cu"]
+SOURCES = ["wf_tables.cu", "wf_api.cu", "wf_server.cu", "wf_mms.cu", "wf_probe.cu", "wf_persist.cu"]
+SOURCES += [f"wf_{part}_p{p}_{t}.cu" for part in ("quad", "lines") for p in (1, 2, 3) for t in ("f32", "f64")]
+SOURCES += [f"wf_persist_p{p}.cu" for p in (1, 2, 3)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 

@@ -14,6 +14,7 @@
 // bands and factors, wind tables, guard flag); kernels address slot z at
 // z * sbytes past slot 0 and skip slots whose active flag is 0, so slots can join and
 // leave between steps without re-capturing the graph.
+#include <limits.h>
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -46,27 +47,16 @@ struct Arena {
     }
 };
 
-// One directional operator of slot 0 (every other slot: same offsets in its block).
-struct Op {
-    bool factored = false;
-    bool compact = false;
-    int mmax = 0;
-    double *band64 = nullptr, *lu64 = nullptr, *spk64 = nullptr, *E64 = nullptr;
-    void *bandP = nullptr, *luP = nullptr, *spkP = nullptr, *EP = nullptr;
-    double *luc64 = nullptr, *spkc64 = nullptr, *Ec64 = nullptr;
-    void *lucP = nullptr, *spkcP = nullptr, *EcP = nullptr;
-    void* fpadP = nullptr;  // compact factors in the line kernels' padded layout (working precision)
-};
-
+// One direction; per-slot pointers are those of slot 0 (every other slot: same offsets in its block).
 struct Dir {
     int n = 0, N = 0;
     double L = 0, h = 0;
-    Chunks ch{};
     // shared by all slots
     double *B64 = nullptr, *D64 = nullptr;
     double *M64 = nullptr, *K64 = nullptr, *G64 = nullptr;
-    // per slot
-    Op op[3];  // 0: M, 1: -theta A (explicit side, band only), 2: M + theta A (implicit side)
+    // per slot: factor tables of M and of the implicit side M + theta A, and (y) the rows of the explicit
+    // operator -theta A
+    void *tabM = nullptr, *tabA = nullptr, *band = nullptr;
 };
 
 // Host-side settings of one slot.
@@ -77,7 +67,7 @@ struct Slot {
     double coef[2][3][3] = {};  // [dir][op][aM, aK, aG]
 };
 
-enum SiteId { S_RHS1, S_X1, S_Y1, S_Y2PRE, S_RHS2, S_X2, S_Y3, S_PERSIST, S_NSITES };
+enum SiteId { S_RHS1, S_X1, S_Y1, S_YMID, S_RHS2, S_X2, S_Y3, S_PERSIST, S_NSITES };
 const char* kSiteNames[S_NSITES] = {"rhs_quadrature_1", "xsolve_1", "ysolve_1", "ysolve_y_substep",
                                     "rhs_quadrature_2", "xsolve_2", "ysolve_2",
                                     "step_persistent"};
@@ -111,14 +101,18 @@ struct wf_handle {
     double* stage = nullptr;   // 2 * Nx * Ny doubles for host transfers
     void* bstage = nullptr;    // whole-batch host transfers (allocated on first use)
     size_t bstage_bytes = 0;
-    double* work64 = nullptr;
-    double* diag = nullptr;    // [4] factorisation diagnostics
     double* wind64 = nullptr;  // staging of wind factors
     int* active_dev = nullptr;
     int* budget_dev = nullptr;  // [S] step budgets (wf_batch_set_budget; -1: unlimited)
     bool budget_on = false;     // some budget was set: the step spends them
     int* status_out = nullptr;  // [S] gathered guard flags
     Dir dx, dy;
+    // chunk length of the line passes; every operator has uniform factors; largest J of the slots' operators,
+    // with exact and with uniform factors
+    int M = 17;
+    bool uni = true;
+    int J[2] = {1, 1};
+    int reach_most[2] = {0, 0};  // rows the states of an operator may reach (0: not set yet)
     // slot blocks: slot-0 pointers, block stride
     int S = 1;
     long long sbytes = 0;
@@ -127,11 +121,10 @@ struct wf_handle {
     bool mms_on = false;       // manufactured-solution forcing (wf_set_mms)
     MmsArgs mms{};
     double* tdev = nullptr;    // device: start time of the next step (advanced only with forcing)
-    int tune[kTune] = {0, 0, 0, 0, 0, 0, 0, 0};  // x lines per CTA (first x pass), y lines per CTA,
-                                           // quadrature segment rows, x lines per warp, x lines
-                                           // per CTA of the second x pass, unused, step form
-                                           // (wf_set_tuning), slots per group of the persistent
-                                           // order (0: the launchers' rules)
+    int tune[kTune] = {0, 0, 0, 0, 0, 0, 0, 0};  // rows per CTA of the first x pass, unused, quadrature
+                                           // segment rows, unused, rows per CTA of the second x
+                                           // pass, unused, step form (wf_set_tuning), slots per
+                                           // group of the persistent order (0: the launchers' rules)
     // persistent step: work items, ticket / abort / item count, arrival counters (allocated on
     // first use); the item list is rebuilt when the active slots or the shapes change
     int4* p_items = nullptr;
@@ -140,7 +133,7 @@ struct wf_handle {
     size_t p_items_cap = 0, p_cnt_cap = 0;
     bool p_dirty = true;
     bool noalloc_run = false;  // wf_step_noalloc in progress: per-pass launches only
-    void *T = nullptr, *phi = nullptr, *Phi = nullptr, *R = nullptr;
+    void *T = nullptr, *phi = nullptr, *Phi = nullptr, *R = nullptr, *W = nullptr;
     int* status = nullptr;
     void* mw = nullptr;  // mean wind (2 values)
     void *fxq = nullptr, *gxq = nullptr, *fyq = nullptr, *gyq = nullptr;
@@ -183,6 +176,8 @@ namespace {
         if (_e != cudaSuccess) return WF_ECUDA; \
     } while (0)
 
+void drop_graphs(wf_handle* h);
+
 size_t esize(int prec) { return prec == WF_FP32 ? 4 : 8; }
 
 template <typename T>
@@ -204,35 +199,15 @@ Batch batch(const wf_handle* h) {
     return b;
 }
 
-// Chunks of length `base`; the last chunk takes the remainder and is merged into its
-// neighbour when it would be shorter than 2p, so every chunk holds at least 2p rows
-// and the interior chunks (1 .. C-2) lie entirely in the Toeplitz part of the operator.
-Chunks make_chunks(int N, int base, int p) {
-    Chunks c;
-    c.N = N;
-    c.base = base;
-    c.C = (N + base - 1) / base;
-    c.last = N - (c.C - 1) * base;
-    if (c.C > 1 && c.last < 2 * p) {
-        c.C -= 1;
-        c.last += base;
-    }
-    if (c.C == 1) c.last = N;
-    return c;
-}
-
 void layout_shared(wf_handle* h, Arena& A) {
     h->stage = A.take<double>(2 * (size_t)h->Nx * h->Ny);
     h->gxi = A.take<double>(16);
     h->gw = A.take<double>(16);
-    h->diag = A.take<double>(4);
     h->active_dev = A.take<int>(h->S);
     h->budget_dev = A.take<int>(h->S);
     h->status_out = A.take<int>(h->S);
     h->tdev = A.take<double>(1);
     const int W = 2 * h->p + 1;
-    const int maxN = h->Nx > h->Ny ? h->Nx : h->Ny;
-    h->work64 = A.take<double>((size_t)maxN * W);
     h->wind64 = A.take<double>((size_t)2 * kMaxRank * (h->Nx + h->Ny));
     Dir* ds[2] = {&h->dx, &h->dy};
     for (Dir* d : ds) {
@@ -245,6 +220,9 @@ void layout_shared(wf_handle* h, Arena& A) {
     }
 }
 
+// Strang / Crank-Nicolson: the middle y pass writes T** to a field of its own
+bool needs_mid(const wf_handle* h) { return h->prm.scheme == WF_STRANG_CN; }
+
 // Slot block, laid out relative to its own start (A.base = start of slot 0).
 void layout_slot(wf_handle* h, Arena& A) {
     const size_t es = esize(h->prec);
@@ -254,39 +232,12 @@ void layout_slot(wf_handle* h, Arena& A) {
     h->Phi = A.take<char>(field * es);
     h->R = A.take<char>(field * es);
     h->status = A.take<int>(4);
-    const int W = 2 * h->p + 1;
-    Dir* ds[2] = {&h->dx, &h->dy};
-    for (Dir* d : ds) {
-        for (Op& o : d->op) {
-            const size_t nE = (size_t)(d->ch.C > 1 ? d->ch.C - 1 : 1) * h->p * h->p;
-            o.mmax = d->ch.base + 2 * h->p;
-            o.band64 = A.take<double>((size_t)d->N * W);
-            o.lu64 = A.take<double>((size_t)d->N * W);
-            o.spk64 = A.take<double>((size_t)d->N * 2 * h->p);
-            o.E64 = A.take<double>(nE);
-            o.luc64 = A.take<double>((size_t)3 * o.mmax * W);
-            o.spkc64 = A.take<double>((size_t)3 * o.mmax * 2 * h->p);
-            o.Ec64 = A.take<double>((size_t)3 * h->p * h->p);
-            if (h->prec == WF_FP32) {
-                o.bandP = A.take<float>((size_t)d->N * W);
-                o.luP = o.factored ? (void*)A.take<float>((size_t)d->N * W) : nullptr;
-                o.spkP = o.factored ? (void*)A.take<float>((size_t)d->N * 2 * h->p) : nullptr;
-                o.EP = o.factored ? (void*)A.take<float>(nE) : nullptr;
-                o.lucP = o.factored ? (void*)A.take<float>((size_t)3 * o.mmax * W) : nullptr;
-                o.spkcP = o.factored ? (void*)A.take<float>((size_t)3 * o.mmax * 2 * h->p) : nullptr;
-                o.EcP = o.factored ? (void*)A.take<float>((size_t)3 * h->p * h->p) : nullptr;
-            } else {
-                o.bandP = o.band64;
-                o.luP = o.lu64;
-                o.spkP = o.spk64;
-                o.EP = o.E64;
-                o.lucP = o.luc64;
-                o.spkcP = o.spkc64;
-                o.EcP = o.Ec64;
-            }
-            o.fpadP = o.factored ? (void*)A.take<char>(fac_pad_elems(h->p, o.mmax) * es) : nullptr;
-        }
+    if (needs_mid(h)) h->W = A.take<char>(field * es);
+    for (Dir* d : {&h->dx, &h->dy}) {
+        d->tabM = A.take<char>(line_tab_bytes(es, h->p, d->N, h->M));
+        d->tabA = A.take<char>(line_tab_bytes(es, h->p, d->N, h->M));
     }
+    if (needs_mid(h)) h->dy.band = A.take<char>((size_t)h->Ny * (2 * h->p + 1) * es);
     const size_t qx = (size_t)kMaxRank * h->nx * h->q, qy = (size_t)kMaxRank * h->ny * h->q;
     h->mw = A.take<char>(2 * es);
     h->fxq = A.take<char>(qx * es);
@@ -360,85 +311,85 @@ int build_tables(wf_handle* h) {
     return WF_OK;
 }
 
-// Bands and chunked factors of every operator of one slot.  Returns WF_OK, WF_ESINGULAR or
-// WF_ETRUNC (neglected spike entries above tol); *worst receives the largest of them.
-int build_factors(wf_handle* h, int slot, double tol, double* worst) {
-    cudaStream_t s = h->stream;
-    const int W = 2 * h->p + 1, S2 = 2 * h->p;
-    *worst = 0.0;
-    Dir* ds[2] = {&h->dx, &h->dy};
-    for (int dd = 0; dd < 2; ++dd) {
-        Dir* d = ds[dd];
-        for (int k = 0; k < 3; ++k) {
-            Op& o = d->op[k];
-            const double* cf = h->slots[slot].coef[dd][k];
-            double zero[4] = {0.0, 0.0, 0.0, 0.0};
-            WF_TRY(cudaMemcpyAsync(h->diag, zero, sizeof(zero), cudaMemcpyHostToDevice, s));
-            WF_TRY(launch_factor(d->M64, d->K64, d->G64, cf[0], cf[1], cf[2], d->N, h->p, d->ch,
-                                 at(h, o.band64, slot), at(h, o.lu64, slot), at(h, o.spk64, slot),
-                                 at(h, o.E64, slot), h->work64, h->diag, s));
-            WF_TRY(launch_compact(at(h, o.lu64, slot), at(h, o.spk64, slot), at(h, o.E64, slot), h->p, d->ch,
-                                  o.mmax, at(h, o.luc64, slot), at(h, o.spkc64, slot), at(h, o.Ec64, slot), h->diag,
-                                  s));
-            double dg[4];
-            WF_TRY(cudaMemcpyAsync(dg, h->diag, sizeof(dg), cudaMemcpyDeviceToHost, s));
-            WF_TRY(cudaStreamSynchronize(s));
-            if (o.factored) {
-                if (dg[0] != 0.0) return WF_ESINGULAR;
-                if (dg[1] > *worst) *worst = dg[1];
-                // every slot must agree on the form the kernels read; slot 0 decides at create
-                if (slot == 0)
-                    o.compact = dg[2] == 0.0;
-                else if (o.compact && dg[2] != 0.0)
-                    return WF_ETRUNC;
-            }
-            if (h->prec != WF_FP32) continue;
-            const size_t nE = (size_t)(d->ch.C > 1 ? d->ch.C - 1 : 1) * h->p * h->p;
-            WF_TRY(launch_to_f32(at(h, o.band64, slot), (float*)at(h, o.bandP, slot), (size_t)d->N * W, s));
-            if (o.factored) {
-                WF_TRY(launch_to_f32(at(h, o.lu64, slot), (float*)at(h, o.luP, slot), (size_t)d->N * W, s));
-                WF_TRY(launch_to_f32(at(h, o.spk64, slot), (float*)at(h, o.spkP, slot), (size_t)d->N * S2, s));
-                WF_TRY(launch_to_f32(at(h, o.E64, slot), (float*)at(h, o.EP, slot), nE, s));
-                WF_TRY(launch_to_f32(at(h, o.luc64, slot), (float*)at(h, o.lucP, slot), (size_t)3 * o.mmax * W, s));
-                WF_TRY(launch_to_f32(at(h, o.spkc64, slot), (float*)at(h, o.spkcP, slot), (size_t)3 * o.mmax * S2,
-                                     s));
-                WF_TRY(launch_to_f32(at(h, o.Ec64, slot), (float*)at(h, o.EcP, slot), (size_t)3 * h->p * h->p, s));
-            }
+// How far the states of an operator's recursions may reach (rows, per direction), decided by the winds of
+// creation: twice the first of these lengths that covers the reach then, no limit for lines shorter than that.
+// The tables hold any reach, but a wind set later that takes a handle far out of the regime it was made for
+// is refused (WF_ETRUNC), and with it a tail of states as long as the line.
+void set_reach_limit(wf_handle* h, const int (&reach)[2]) {
+    const int rows32[] = {32, 48, 64, 96, 128, 256, 512, 1024, 2048, 8192};
+    const int rows64[] = {48, 64, 96, 128, 192, 256, 512, 1024, 2048, 8192};
+    const int N[2] = {h->Nx, h->Ny};
+    for (int b : h->prec == WF_FP32 ? rows32 : rows64) {
+        bool covered = true;
+        for (int d = 0; d < 2; ++d) {
+            const int rows = 2 * std::max(b, (N[d] + 31) / 32);
+            h->reach_most[d] = N[d] < rows ? INT_MAX : rows + h->M;
+            covered = covered && reach[d] <= h->reach_most[d] / 2;
         }
+        if (covered) return;
     }
-    for (Dir* d : ds)
-        for (Op& o : d->op)
-            if (o.factored)
-                WF_TRY(launch_pad_factors(h->prec, h->p, o.mmax, at(h, o.lucP, slot), at(h, o.spkcP, slot),
-                                          at(h, o.EcP, slot), at(h, o.fpadP, slot), s));
-    const Slot& sl = h->slots[slot];
-    if (h->prec == WF_FP32) {
-        const float b[2] = {(float)sl.wind_x, (float)sl.wind_y};
-        WF_TRY(cudaMemcpyAsync(at(h, h->mw, slot), b, sizeof(b), cudaMemcpyHostToDevice, s));
-        WF_TRY(cudaStreamSynchronize(s));  // b goes out of scope
-    } else {
-        const double b[2] = {sl.wind_x, sl.wind_y};
-        WF_TRY(cudaMemcpyAsync(at(h, h->mw, slot), b, sizeof(b), cudaMemcpyHostToDevice, s));
-        WF_TRY(cudaStreamSynchronize(s));
-    }
-    return *worst > tol ? WF_ETRUNC : WF_OK;
+    h->reach_most[0] = h->reach_most[1] = INT_MAX;
 }
 
-double trunc_tol(const wf_handle* h) { return h->prec == WF_FP32 ? 1e-8 : 1e-15; }
-
-FactorV fv(const Op& o, const Chunks& ch) {
-    FactorV f;
-    f.ch = ch;
-    f.lu = o.luP;
-    f.spk = o.spkP;
-    f.E = o.EP;
-    f.compact = o.compact ? 1 : 0;
-    f.mmax = o.mmax;
-    f.luc = o.lucP;
-    f.spkc = o.spkcP;
-    f.Ec = o.EcP;
-    f.fpad = o.compact ? o.fpadP : nullptr;
-    return f;
+// Factor tables of the operators of slots slot .. slot + count - 1 (those of `slot`; each slot has its own
+// copy) and their mean wind.  Returns WF_OK, WF_ESINGULAR or WF_ETRUNC (set_reach_limit).
+int build_factors(wf_handle* h, int slot, int count) {
+    cudaStream_t s = h->stream;
+    const Slot& sl = h->slots[slot];
+    TabJobs jobs;
+    memset(&jobs, 0, sizeof(jobs));
+    Dir* ds[2] = {&h->dx, &h->dy};
+    auto add = [&](int dd, int k, void* out, int band) {
+        const Dir* d = ds[dd];
+        const double* cf = sl.coef[dd][k];
+        TabJob& j = jobs.job[jobs.n++];
+        j.M = d->M64;
+        j.K = d->K64;
+        j.G = d->G64;
+        j.aM = cf[0];
+        j.aK = cf[1];
+        j.aG = cf[2];
+        j.N = d->N;
+        j.chunk = h->M;
+        j.out = out;
+        j.band = band;
+    };
+    for (int dd = 0; dd < 2; ++dd) {
+        add(dd, 0, at(h, ds[dd]->tabM, slot), 0);
+        add(dd, 2, at(h, ds[dd]->tabA, slot), 0);
+    }
+    if (needs_mid(h)) add(1, 1, at(h, h->dy.band, slot), 1);
+    jobs.mw = at(h, h->mw, slot);
+    jobs.wind_x = sl.wind_x;
+    jobs.wind_y = sl.wind_y;
+    jobs.tol = h->prec == WF_FP32 ? 1e-8 : 1e-15;
+    jobs.slots = count;
+    jobs.sbytes = h->sbytes;
+    WF_TRY(launch_line_tables(h->prec, h->p, jobs, s));
+    int hdr[4][4];
+    for (int k = 0; k < 4; ++k)
+        WF_TRY(cudaMemcpyAsync(hdr[k], jobs.job[k].out, sizeof(hdr[k]), cudaMemcpyDeviceToHost, s));
+    WF_TRY(cudaStreamSynchronize(s));
+    bool uni = h->uni;
+    int reach[2] = {0, 0};
+    for (int k = 0; k < 4; ++k) {
+        if (hdr[k][3]) return WF_ESINGULAR;
+        uni = uni && hdr[k][0] == 1;
+        reach[k / 2] = std::max(reach[k / 2], hdr[k][hdr[k][0] == 1 ? 1 : 2] * h->M);
+    }
+    if (h->reach_most[0] == 0) set_reach_limit(h, reach);
+    if (reach[0] > h->reach_most[0] || reach[1] > h->reach_most[1]) return WF_ETRUNC;
+    int J[2] = {h->J[0], h->J[1]};
+    for (int k = 0; k < 4; ++k)
+        for (int q = 0; q < 2; ++q)
+            if (q == 0 || hdr[k][0] == 1) J[q] = std::max(J[q], hdr[k][2 - q]);
+    if (J[0] != h->J[0] || J[1] != h->J[1] || uni != h->uni) {
+        h->uni = uni;
+        h->J[0] = J[0];
+        h->J[1] = J[1];
+        drop_graphs(h);  // the tiles of a y pass reach J chunks past their own
+    }
+    return WF_OK;
 }
 
 cudaEvent_t take_event(wf_handle* h) {
@@ -504,28 +455,37 @@ LineArgs line_args(wf_handle* h, int xsite) {
     const bool xdir = xsite != 0;
     LineArgs a;
     memset(&a, 0, sizeof(a));
+    a.N = xdir ? h->Nx : h->Ny;
+    a.M = h->M;
+    a.C = line_chunks(a.N, a.M);
+    a.uni = h->uni ? 1 : 0;
+    a.J = h->uni ? h->J[1] : std::max(h->J[0], h->J[1]);
     a.nlines = xdir ? h->Ny : h->Nx;
-    a.G = xsite == 1 ? h->tune[0] : (xsite == 2 ? h->tune[4] : h->tune[1]);
-    a.rpw = xdir ? h->tune[3] : 0;
+    a.G = xsite == 1 ? h->tune[0] : (xsite == 2 ? h->tune[4] : 0);
     a.pitch = h->pitch;
     a.tmax = kTmax;
     a.tstatus = h->status;
     a.wait_ns = h->wait_ns;
-    // every y pass of a step reads a right-hand side that the step writes again before its next use
-    a.in_dead = xdir ? 0 : 1;
     a.b = batch(h);
     return a;
 }
 
-void add_line(LineArgs& a, const void* in, void* out, const Op& o, const Chunks& ch, const void* base = nullptr,
-              const void* premul = nullptr, double prescale = 1.0) {
+void add_line(LineArgs& a, const void* in, void* out, const void* tab, const void* base = nullptr) {
     a.in[a.narr] = in;
     a.out[a.narr] = out;
-    a.f[a.narr] = fv(o, ch);
+    a.tab[a.narr] = tab;
     a.base[a.narr] = base;
-    a.premul[a.narr] = premul;
-    a.prescale[a.narr] = prescale;
     a.narr++;
+}
+
+cudaError_t launch_lines(const wf_handle* h, int kind, const LineArgs& a) {
+    const bool f32 = h->prec == WF_FP32;
+    switch (h->p) {
+        case 1: return f32 ? launch_lines_p1_f32(kind, a, h->stream) : launch_lines_p1_f64(kind, a, h->stream);
+        case 2: return f32 ? launch_lines_p2_f32(kind, a, h->stream) : launch_lines_p2_f64(kind, a, h->stream);
+        case 3: return f32 ? launch_lines_p3_f32(kind, a, h->stream) : launch_lines_p3_f64(kind, a, h->stream);
+    }
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t upload_active(wf_handle* h) {
@@ -568,7 +528,6 @@ cudaError_t rhs_and_forcing(wf_handle* h, const RhsArgs& r) {
 }
 
 cudaError_t enqueue_step_body(wf_handle* h);
-void drop_graphs(wf_handle* h);
 
 // The persistent form (one quadrature launch, then one launch over every line pass of every active
 // slot) takes PR with one F per step; tuning value 6 picks it (2) or the per-pass launches (1,
@@ -577,28 +536,21 @@ bool use_persist(const wf_handle* h) {
     // (a launch over a group of slots, gn > 0, takes the per-pass form: the persistent plan lists
     // every active slot of the handle)
     if (h->noalloc_run || h->gn > 0 || h->prm.scheme != WF_PR || h->prm.F_timing != WF_F_ONCE) return false;
-    if (!persist_supported(h->prec, h->p, h->wr)) return false;
     return h->tune[6] == 2;
 }
 
 // Arguments of the persistent step: those of the per-pass launches of the same step.
 void persist_args(wf_handle* h, PersistHost* ph) {
-    Op* X = h->dx.op;
-    Op* Y = h->dy.op;
-    const Chunks& cx = h->dx.ch;
-    const Chunks& cy = h->dy.ch;
     memset(ph, 0, sizeof(*ph));
     ph->prec = h->prec;
     ph->p = h->p;
     ph->x = line_args(h, 1);
-    add_line(ph->x, h->R, h->R, X[2], cx);
-    add_line(ph->x, h->Phi, h->Phi, X[0], cx);
+    add_line(ph->x, h->R, h->R, h->dx.tabA);
+    add_line(ph->x, h->Phi, h->Phi, h->dx.tabM);
     ph->y = line_args(h, 0);
-    add_line(ph->y, h->R, h->T, Y[2], cy, h->T);
-    add_line(ph->y, h->Phi, h->phi, Y[0], cy, h->phi);
+    add_line(ph->y, h->R, h->T, h->dy.tabA, h->T);
+    add_line(ph->y, h->Phi, h->phi, h->dy.tabM, h->phi);
     ph->y.status = h->status;
-    ph->xG = h->tune[0];
-    ph->yG = h->tune[1];
     ph->nslots_cap = h->S;
     ph->wait_ns = h->wait_ns;
     ph->status = h->status;
@@ -736,113 +688,90 @@ cudaError_t enqueue_steps(wf_handle* h, int n) {
 
 cudaError_t enqueue_step_body(wf_handle* h) {
     cudaStream_t s = h->stream;
-    const int prec = h->prec, p = h->p;
-    Op* X = h->dx.op;
-    Op* Y = h->dy.op;
-    const Chunks& cx = h->dx.ch;
-    const Chunks& cy = h->dy.ch;
+    const Dir &X = h->dx, &Y = h->dy;
     cudaError_t e;
+    auto quad = [&](int site, const RhsArgs& r) {
+        if ((e = timed(h, site, [&] { return rhs_and_forcing(h, r); })) != cudaSuccess) return false;
+        if (site == S_RHS1 && h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return false;
+        return true;
+    };
+    auto lines = [&](int site, int kind, const LineArgs& a) {
+        return (e = timed(h, site, [&] { return launch_lines(h, kind, a); })) == cudaSuccess;
+    };
+    // x pass of the increment's right-hand side with `tab` and of the fuel increment
+    auto x_pass = [&](int site, const void* tab, bool fuel) {
+        LineArgs a = line_args(h, site == S_X2 ? 2 : 1);
+        add_line(a, h->R, h->R, tab);
+        if (fuel) add_line(a, h->Phi, h->Phi, X.tabM);
+        return lines(site, 0, a);
+    };
+    // y pass: T = base + solution with `tab`; last: the fuel too, and the guard on T
+    auto y_pass = [&](int site, const void* tab, const void* base, bool last) {
+        LineArgs a = line_args(h, 0);
+        add_line(a, h->R, h->T, tab, base);
+        if (last) {
+            add_line(a, h->Phi, h->phi, Y.tabM, h->phi);
+            a.status = h->status;
+        }
+        return lines(site, 1, a);
+    };
+    const double tau = h->dt, half = 0.5 * h->dt;
     if (h->prm.scheme == WF_EXPLICIT) {
         // (M^x (x) M^y)(T^{n+1} - T^n) = tau F - tau (A_x (x) M^y) T^n - tau (M^x (x) A_y) T^n
-        RhsArgs r1 = rhs_args(h, h->Phi, h->R, h->dt, false);
-        auto l1 = [&] { return rhs_and_forcing(h, r1); };
-        if ((e = timed(h, S_RHS1, l1)) != cudaSuccess) return e;
-        if (h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return e;
-        LineArgs x1 = line_args(h, 1);
-        add_line(x1, h->R, h->R, X[0], cx);
-        add_line(x1, h->Phi, h->Phi, X[0], cx);
-        if ((e = timed(h, S_X1, [&] { return launch_xsolve(prec, p, x1, s); })) != cudaSuccess) return e;
-        LineArgs y1 = line_args(h, 0);
-        add_line(y1, h->R, h->T, Y[0], cy, h->T);
-        add_line(y1, h->Phi, h->phi, Y[0], cy, h->phi);
-        y1.status = h->status;
-        if ((e = timed(h, S_Y3, [&] { return launch_ysolve(prec, p, y1, s); })) != cudaSuccess) return e;
-        return cudaSuccess;
+        quad(S_RHS1, rhs_args(h, h->Phi, h->R, tau, false)) && x_pass(S_X1, X.tabM, true) &&
+            y_pass(S_Y3, Y.tabM, h->T, true);
+        return e;
     }
     if (h->prm.scheme == WF_PR && h->prm.F_timing == WF_F_ONCE) {
         // X_+ lines along x, Y_+ along y.  Step form 1: a launch per array and per kind of strip
-        RhsArgs r1 = rhs_args(h, h->Phi, h->R, h->dt, false);
+        RhsArgs r1 = rhs_args(h, h->Phi, h->R, tau, false);
         const bool pers = use_persist(h) && h->p_ctl;
         const bool split = h->tune[6] == 1 || (h->tune[6] == 3 && h->gn == 0);
         r1.parts = split ? 1 : 0;
-        auto l1 = [&] { return rhs_and_forcing(h, r1); };
-        if ((e = timed(h, S_RHS1, l1)) != cudaSuccess) return e;
-        if (h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return e;
+        if (!quad(S_RHS1, r1)) return e;
         if (pers) {
             PersistHost ph;
             persist_args(h, &ph);
             return timed(h, S_PERSIST, [&] { return persist_step(ph, nullptr, true, s); });
         }
-        for (int part = 0; part < (split ? 2 : 1); ++part) {
-            LineArgs x1 = line_args(h, 1);
-            if (part == 0) add_line(x1, h->R, h->R, X[2], cx);
-            if (part == 1 || !split) add_line(x1, h->Phi, h->Phi, X[0], cx);
-            if ((e = timed(h, S_X1, [&] { return launch_xsolve(prec, p, x1, s); })) != cudaSuccess) return e;
+        if (!split) {
+            x_pass(S_X1, X.tabA, true) && y_pass(S_Y1, Y.tabA, h->T, true);
+            return e;
         }
-        for (int part = 0; part < (split ? 2 : 1); ++part) {
-            LineArgs y1 = line_args(h, 0);
-            if (part == 0) add_line(y1, h->R, h->T, Y[2], cy, h->T);
-            if (part == 1 || !split) add_line(y1, h->Phi, h->phi, Y[0], cy, h->phi);
-            if (part == 0) y1.status = h->status;  // the guard watches T
-            if ((e = timed(h, S_Y1, [&] { return launch_ysolve(prec, p, y1, s); })) != cudaSuccess) return e;
-        }
-        return cudaSuccess;
+        LineArgs a = line_args(h, 1);
+        add_line(a, h->R, h->R, X.tabA);
+        if (!lines(S_X1, 0, a)) return e;
+        a = line_args(h, 1);
+        add_line(a, h->Phi, h->Phi, X.tabM);
+        if (!lines(S_X1, 0, a)) return e;
+        a = line_args(h, 0);
+        add_line(a, h->R, h->T, Y.tabA, h->T);
+        a.status = h->status;
+        if (!lines(S_Y1, 1, a)) return e;
+        a = line_args(h, 0);
+        add_line(a, h->Phi, h->phi, Y.tabM, h->phi);
+        lines(S_Y1, 1, a);
+        return e;
     }
     if (h->prm.scheme == WF_PR) {
         // F re-evaluated at T* in the second substep
-        const double th = 0.5 * h->dt;
-        RhsArgs r1 = rhs_args(h, h->Phi, h->R, th, false);
-        auto l1 = [&] { return rhs_and_forcing(h, r1); };
-        if ((e = timed(h, S_RHS1, l1)) != cudaSuccess) return e;
-        if (h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return e;
-        LineArgs x1 = line_args(h, 1);
-        add_line(x1, h->R, h->R, X[2], cx);
-        add_line(x1, h->Phi, h->Phi, X[0], cx);
-        if ((e = timed(h, S_X1, [&] { return launch_xsolve(prec, p, x1, s); })) != cudaSuccess) return e;
-        LineArgs y1 = line_args(h, 0);
-        add_line(y1, h->R, h->T, Y[0], cy, h->T);
-        if ((e = timed(h, S_Y1, [&] { return launch_ysolve(prec, p, y1, s); })) != cudaSuccess) return e;
-        RhsArgs r2 = rhs_args(h, nullptr, h->R, th, false);
-        auto l2 = [&] { return rhs_and_forcing(h, r2); };
-        if ((e = timed(h, S_RHS2, l2)) != cudaSuccess) return e;
-        LineArgs x2 = line_args(h, 2);
-        add_line(x2, h->R, h->R, X[0], cx);
-        if ((e = timed(h, S_X2, [&] { return launch_xsolve(prec, p, x2, s); })) != cudaSuccess) return e;
-        LineArgs y2 = line_args(h, 0);
-        add_line(y2, h->R, h->T, Y[2], cy, h->T);
-        add_line(y2, h->Phi, h->phi, Y[0], cy, h->phi);
-        y2.status = h->status;
-        if ((e = timed(h, S_Y3, [&] { return launch_ysolve(prec, p, y2, s); })) != cudaSuccess) return e;
-        return cudaSuccess;
+        quad(S_RHS1, rhs_args(h, h->Phi, h->R, half, false)) && x_pass(S_X1, X.tabA, true) &&
+            y_pass(S_Y1, Y.tabM, h->T, false) && quad(S_RHS2, rhs_args(h, nullptr, h->R, half, false)) &&
+            x_pass(S_X2, X.tabM, false) && y_pass(S_Y3, Y.tabA, h->T, true);
+        return e;
     }
-    // Strang / Crank-Nicolson
-    const double half = 0.5 * h->dt;
-    RhsArgs r1 = rhs_args(h, h->Phi, h->R, half, true);
-    auto l1 = [&] { return rhs_and_forcing(h, r1); };
-    if ((e = timed(h, S_RHS1, l1)) != cudaSuccess) return e;
-    if (h->ev_rhs && (e = cudaEventRecord(h->ev_rhs, s)) != cudaSuccess) return e;
-    LineArgs x1 = line_args(h, 1);
-    add_line(x1, h->R, h->R, X[2], cx);
-    add_line(x1, h->Phi, h->Phi, X[0], cx);
-    if ((e = timed(h, S_X1, [&] { return launch_xsolve(prec, p, x1, s); })) != cudaSuccess) return e;
-    LineArgs y1 = line_args(h, 0);
-    add_line(y1, h->R, h->T, Y[0], cy, h->T);
-    if ((e = timed(h, S_Y1, [&] { return launch_ysolve(prec, p, y1, s); })) != cudaSuccess) return e;
-    LineArgs yy = line_args(h, 0);
-    add_line(yy, h->T, h->T, Y[2], cy, h->T, Y[1].bandP, 2.0);
-    if ((e = timed(h, S_Y2PRE, [&] { return launch_ysolve(prec, p, yy, s); })) != cudaSuccess) return e;
+    // Strang / Crank-Nicolson: the middle y pass (first substep's y solve and the y substep in one) leaves
+    // T** in W
+    if (!quad(S_RHS1, rhs_args(h, h->Phi, h->R, half, true)) || !x_pass(S_X1, X.tabA, true)) return e;
+    LineArgs a = line_args(h, 0);
+    add_line(a, h->R, h->W, Y.tabM, h->T);
+    a.tab[1] = Y.tabA;
+    a.band = Y.band;
+    if (!lines(S_YMID, 2, a)) return e;
     RhsArgs r2 = rhs_args(h, nullptr, h->R, half, true);
-    auto l2 = [&] { return rhs_and_forcing(h, r2); };
-    if ((e = timed(h, S_RHS2, l2)) != cudaSuccess) return e;
-    LineArgs x2 = line_args(h, 2);
-    add_line(x2, h->R, h->R, X[2], cx);
-    if ((e = timed(h, S_X2, [&] { return launch_xsolve(prec, p, x2, s); })) != cudaSuccess) return e;
-    LineArgs y2 = line_args(h, 0);
-    add_line(y2, h->R, h->T, Y[0], cy, h->T);
-    add_line(y2, h->Phi, h->phi, Y[0], cy, h->phi);
-    y2.status = h->status;
-    if ((e = timed(h, S_Y3, [&] { return launch_ysolve(prec, p, y2, s); })) != cudaSuccess) return e;
-    return cudaSuccess;
+    r2.T = h->W;
+    quad(S_RHS2, r2) && x_pass(S_X2, X.tabA, false) && y_pass(S_Y3, Y.tabM, h->W, true);
+    return e;
 }
 
 void drop_graphs(wf_handle* h) {
@@ -1033,23 +962,15 @@ bool create_args_ok(int nx, int ny, int p, double dt, const wf_params* params, i
     return params_ok(*params);
 }
 
-// Chunk lengths tried at creation, shortest first: the truncated reduced system must neglect spike
-// entries below 1e-8 (FP32) or 1e-15 (FP64), and the shortest length that does is kept.
-constexpr int kBaseTries = 10;
-const int kBases32[kBaseTries] = {32, 48, 64, 96, 128, 256, 512, 1024, 2048, 8192};
-const int kBases64[kBaseTries] = {48, 64, 96, 128, 192, 256, 512, 1024, 2048, 8192};
-
-// Chunks of both directions for creation attempt `attempt`: at most 32 chunks per line (one warp
-// lane or one thread row each); odd lengths keep the 32 lanes of the x pass on distinct banks.
-void set_chunks(wf_handle* h, int attempt) {
-    const int* bases = h->prec == WF_FP32 ? kBases32 : kBases64;
-    for (Dir* d : {&h->dx, &h->dy}) {
-        int base = bases[attempt];
-        const int need = (d->N + 31) / 32;
-        if (base < need) base = need;
-        base |= 1;
-        d->ch = make_chunks(d->N, base, h->p);
-    }
+// Chunk length of the line passes (values per thread), by the longest line alone, so that a scenario's bits do
+// not depend on the batch it runs in.  Short chunks spread a small domain over more threads, long ones waste
+// less on states and halos.  us per step at 9 / 17 / 33: 130^2 FP32 25 / 29 / 35 (sum of its launches),
+// 258^2 x 256 368 / 321 / 354, 515^2 cubic x 8 110 / 105 / 105, 1026^2 34 / 35.5 / 37, 4099^2 cubic 617 / 554 / 538;
+// FP64: 66^2 75 / 81 / 100, 1026^2 749 / 698 / 745.
+int chunk_rule(int prec, int Nx, int Ny) {
+    const int N = std::max(Nx, Ny);
+    if (N <= 144) return 9;
+    return N <= (prec == WF_FP32 ? 1600 : 1088) ? 17 : 33;
 }
 
 // Shared-region and per-slot byte counts of the handle's layout for its current chunks.
@@ -1084,8 +1005,7 @@ void init_fields(wf_handle* h, int nx, int ny, int p, double dt, const wf_params
     h->dy.N = h->Ny;
     h->dy.L = params->Ly;
     h->dy.h = params->Ly / ny;
-    for (Dir* d : {&h->dx, &h->dy})
-        for (int k = 0; k < 3; ++k) d->op[k].factored = (k != 1);
+    h->M = chunk_rule(h->prec, h->Nx, h->Ny);
 }
 
 }  // namespace
@@ -1094,15 +1014,10 @@ int wf_batch_bytes(int nx, int ny, int p, double dt, const wf_params* params, in
     if (!bytes || !create_args_ok(nx, ny, p, dt, params, capacity)) return WF_EINVAL;
     wf_handle h;
     init_fields(&h, nx, ny, p, dt, params, capacity);
-    size_t most = 0;
-    for (int attempt = 0; attempt < kBaseTries; ++attempt) {
-        set_chunks(&h, attempt);
-        size_t shared = 0;
-        long long sb = 0;
-        layout_sizes(&h, &shared, &sb);
-        most = std::max(most, shared + (size_t)sb * capacity + 256);
-    }
-    *bytes = most;
+    size_t shared = 0;
+    long long sb = 0;
+    layout_sizes(&h, &shared, &sb);
+    *bytes = shared + (size_t)sb * capacity + 256;
     return WF_OK;
 }
 
@@ -1135,46 +1050,27 @@ int wf_batch_create(int nx, int ny, int p, double dt, const wf_params* params, i
     }
     h->stream = h->own;
 
-    // Chunk length: the shortest of the tried lengths whose neglected spike entries stay below
-    // the truncation tolerance (for the creation wind).
-    const double tol = trunc_tol(h);
     int rc = WF_OK;
     size_t shared = 0;
-    for (int attempt = 0; attempt < kBaseTries; ++attempt) {
-        set_chunks(h, attempt);
-        if (h->mem) {
-            cudaFree(h->mem);
-            h->mem = nullptr;
-        }
-        layout_sizes(h, &shared, &h->sbytes);
-        h->mem_bytes = shared + (size_t)h->sbytes * capacity + 256;
-        if (cudaMalloc(&h->mem, h->mem_bytes) != cudaSuccess) {
-            destroy(h);
-            return WF_ENOMEM;
-        }
-        Arena A2;
-        A2.base = reinterpret_cast<char*>(h->mem);
-        layout_shared(h, A2);
-        Arena B2;
-        B2.base = reinterpret_cast<char*>(h->mem) + shared;
-        h->slots_mem = B2.base;
-        layout_slot(h, B2);
-        // every slot block starts zeroed (fields, guard flags, unused wind ranks); no budgets
-        if (cudaMemsetAsync(B2.base, 0, (size_t)h->sbytes * capacity, h->stream) != cudaSuccess ||
-            cudaMemsetAsync(h->budget_dev, 0xff, sizeof(int) * capacity, h->stream) != cudaSuccess) {
-            rc = WF_ECUDA;
-            break;
-        }
-        if ((rc = build_tables(h)) != WF_OK) break;
-        double worst = 0.0;
-        rc = build_factors(h, 0, tol, &worst);
-        if (rc != WF_ETRUNC) break;
-        if (h->dx.ch.C == 1 && h->dy.ch.C == 1) break;
+    layout_sizes(h, &shared, &h->sbytes);
+    h->mem_bytes = shared + (size_t)h->sbytes * capacity + 256;
+    if (cudaMalloc(&h->mem, h->mem_bytes) != cudaSuccess) {
+        destroy(h);
+        return WF_ENOMEM;
     }
-    for (int sl = 1; sl < capacity && rc == WF_OK; ++sl) {
-        double worst = 0.0;
-        rc = build_factors(h, sl, tol, &worst);
-    }
+    Arena A2;
+    A2.base = reinterpret_cast<char*>(h->mem);
+    layout_shared(h, A2);
+    Arena B2;
+    B2.base = reinterpret_cast<char*>(h->mem) + shared;
+    h->slots_mem = B2.base;
+    layout_slot(h, B2);
+    // every slot block starts zeroed (fields, guard flags, unused wind ranks); no budgets
+    if (cudaMemsetAsync(B2.base, 0, (size_t)h->sbytes * capacity, h->stream) != cudaSuccess ||
+        cudaMemsetAsync(h->budget_dev, 0xff, sizeof(int) * capacity, h->stream) != cudaSuccess)
+        rc = WF_ECUDA;
+    if (rc == WF_OK) rc = build_tables(h);
+    if (rc == WF_OK) rc = build_factors(h, 0, capacity);
     if (rc == WF_OK && (upload_active(h) != cudaSuccess || cudaStreamSynchronize(h->stream) != cudaSuccess))
         rc = WF_ECUDA;
     if (rc != WF_OK) {
@@ -1224,14 +1120,13 @@ int wf_set_mean_wind(wf_handle* h, int slot, double wind_x, double wind_y) {
     sl.wind_x = wind_x;
     sl.wind_y = wind_y;
     set_slot_coeffs(h, sl);
-    double worst = 0.0;
-    int rc = build_factors(h, slot, trunc_tol(h), &worst);
+    int rc = build_factors(h, slot, 1);
     if (rc != WF_OK) {
         // keep the slot usable: back to the previous wind (whose factors were valid)
         sl.wind_x = old_x;
         sl.wind_y = old_y;
         set_slot_coeffs(h, sl);
-        const int rc2 = build_factors(h, slot, trunc_tol(h), &worst);
+        const int rc2 = build_factors(h, slot, 1);
         return rc2 == WF_OK ? rc : rc2;
     }
     if (h->mms_on && slot == 0) {
@@ -1253,8 +1148,7 @@ int wf_batch_set_slot(wf_handle* h, int slot, const double* T, const double* fue
         sl.wind_x = wind_x;
         sl.wind_y = wind_y;
         set_slot_coeffs(h, sl);
-        double worst = 0.0;
-        const int rc = build_factors(h, slot, trunc_tol(h), &worst);
+        const int rc = build_factors(h, slot, 1);
         if (rc != WF_OK) return rc;
     }
     int rc = set_slot_wind_factors(h, slot, wind_rank, wind_factors);
@@ -1619,8 +1513,7 @@ int wf_autotune(wf_handle* h, int reps) {
     // values between the powers of two: the number of (strip, segment) work items against
     // the resident warps decides how full the last wave is.
     static const int kSeg[] = {0, 128, 96, 80, 64, 56, 48, 40, 32, 28, 24, 21, 20, 16, 12};
-    static const int kLines[] = {0, 32, 16, 8, 4, 2, 1};
-    static const int kRpw[] = {0, 1, 2, 4};
+    static const int kLines[] = {0, 8, 4, 2, 1};
     static const int kModeAll[] = {0, 2, 3};  // the rule, persistent, two slot groups
     static const int kGroup[] = {0, 1, 2, 4, 8, 16, 32, 64};
     struct Axis {
@@ -1628,8 +1521,7 @@ int wf_autotune(wf_handle* h, int reps) {
         const int* v;
         int n;
     };
-    const bool pers = persist_supported(h->prec, h->p, h->wr) && h->prm.scheme == WF_PR &&
-                      h->prm.F_timing == WF_F_ONCE;
+    const bool pers = h->prm.scheme == WF_PR && h->prm.F_timing == WF_F_ONCE;
     const bool grp = h->S >= 2 && !h->mms_on;
     // only Strang / Crank-Nicolson and F per substep have a second x pass
     const bool second_x = h->prm.scheme == WF_STRANG_CN ||
@@ -1641,8 +1533,6 @@ int wf_autotune(wf_handle* h, int reps) {
     // the persistent form's group size; the second sweep refines the shapes under the chosen form
     const Axis order[] = {{2, kSeg, (int)(sizeof(kSeg) / sizeof(int))},
                           {0, kLines, (int)(sizeof(kLines) / sizeof(int))},
-                          {3, kRpw, (int)(sizeof(kRpw) / sizeof(int))},
-                          {1, kLines, (int)(sizeof(kLines) / sizeof(int))},
                           {4, kLines, second_x ? (int)(sizeof(kLines) / sizeof(int)) : 0},
                           {6, kMode, nMode > 1 ? nMode : 0},
                           {7, kGroup, pers && h->S > 1 ? (int)(sizeof(kGroup) / sizeof(int)) : 0}};
@@ -1818,13 +1708,13 @@ int wf_set_tuning(wf_handle* h, const int* shape) {
 
 // ---- allocation-free step ------------------------------------------------------------
 //
-// Scratch of wf_step_noalloc: the two intermediate fields of a step (Phi, R), each at
-// most kNoallocMaxElems padded FP32 coefficients, in one array that every GPU loading
-// this library holds until the process exits (4 MiB).  Host code must not hand the
+// Scratch of wf_step_noalloc: the three intermediate fields of a step (Phi, R and, for Strang
+// splitting, T**), each at most kNoallocMaxElems padded FP32 coefficients, in one array that
+// every GPU loading this library holds until the process exits (6 MiB).  Host code must not hand the
 // symbol itself to a kernel: on the host it names a host-side placeholder.  Its device
 // address is looked up once per device with cudaGetSymbolAddress and cached.
 constexpr size_t kNoallocMaxElems = size_t(1) << 19;
-static __device__ __align__(256) float g_noalloc_scratch[2 * kNoallocMaxElems];
+static __device__ __align__(256) float g_noalloc_scratch[3 * kNoallocMaxElems];
 
 namespace {
 constexpr int kNoallocMaxDevices = 64;
@@ -1864,12 +1754,13 @@ extern "C" int wf_step_noalloc(wf_handle* h, void* T, void* fuel, int pitch, int
     // Run the handle's own step sequence with the caller's state and the static scratch in
     // place of the handle's buffers.  Every scratch element a kernel reads was written earlier
     // in the same step, so nothing needs clearing between calls.
-    void* save[4] = {h->T, h->phi, h->Phi, h->R};
+    void* save[5] = {h->T, h->phi, h->Phi, h->R, h->W};
     const int save_pitch = h->pitch;
     h->T = T;
     h->phi = fuel;
     h->Phi = scratch;
     h->R = scratch + kNoallocMaxElems;
+    h->W = scratch + 2 * kNoallocMaxElems;
     h->pitch = pitch;
     cudaError_t e = cudaSuccess;
     h->noalloc_run = true;  // the persistent step's buffers may not exist yet: per-pass launches
@@ -1879,6 +1770,7 @@ extern "C" int wf_step_noalloc(wf_handle* h, void* T, void* fuel, int pitch, int
     h->phi = save[1];
     h->Phi = save[2];
     h->R = save[3];
+    h->W = save[4];
     h->pitch = save_pitch;
     return e == cudaSuccess ? WF_OK : WF_ECUDA;
 }

@@ -8,7 +8,7 @@
 //     derivative D[e][a][l], e < n, a < q = p+1, l <= p;
 //   - 1-D banded matrices: band[r][d] = A[r][r+d-p], d in [0, 2p], zero
 //     outside the matrix;
-//   - chunked LU factors of a 1-D operator (see Factor below).
+//   - LU factors of a 1-D operator (see the factor tables below).
 #pragma once
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -52,46 +52,47 @@ struct Phys {
     int heat_by_fuel;
 };
 
-// Partition of a line of N unknowns into C chunks: chunk k starts at k*base and has
-// length base, except the last one, which has length `last` in [2p, base + 2p)
-// (a single chunk, C = 1, has length N).
-struct Chunks {
-    int N, C, base, last;
-};
-__host__ __device__ inline int chunk_start(const Chunks& c, int k) { return k * c.base; }
-__host__ __device__ inline int chunk_len(const Chunks& c, int k) { return k < c.C - 1 ? c.base : c.last; }
-__host__ __device__ inline int chunk_of(const Chunks& c, int x) {
-    const int k = x / c.base;
-    return k < c.C - 1 ? k : c.C - 1;
+// ---- factor tables of the line solves ------------------------------------------------
+// A line of N unknowns is cut into C = ceil(N / M) chunks of M (the last one padded).  The table of one
+// operator A = aM M + aK K + aG G (half-bandwidth p), written once per operator in the working precision from
+// FP64 LU factors without pivoting (wf_lines.cuh has the method):
+//   header (kTabHeader bytes of ints): [0] 1: uniform factors and end corrections, 0: exact factors of every
+//     row; [1] J, the chunks whose states a chunk's entering state takes in, with uniform factors, [2] with
+//     exact ones; [3] 1 if a pivot was below 1e-300 ||A||
+//   l[4], u[4]                uniform rows of F and U
+//   Tf[p][p], Tb[p][p]        transfer of a state (the last p values of a forward, the first p of a backward
+//                             recursion, nearest first) through a chunk of uniform rows
+//   VT[kEndRows + M][V], VB[kEndRows + 2M][V]  (V = 2, 4, 8) end corrections of the first J and last J + 1 chunks
+//   F[C*M][p (4 for p = 3)]   multipliers: row r subtracts F[r][i-1] * y[r-i], i = 1..p
+//   U[C*M][2 (p = 1) or 4]    1 / u_rr, then u_r,r+j / u_rr, j = 1..p
+//   Pf[C][p][p], Pb[C][p][p]  transfers through every chunk
+// every part rounded up to a multiple of four elements.
+constexpr int kTabHeader = 64;
+constexpr int kEndRows = 128;  // J * M at most for the uniform form
+__host__ __device__ constexpr int tab_round(int n) { return (n + 3) & ~3; }
+inline int line_chunks(int N, int M) { return (N + M - 1) / M; }
+inline size_t line_tab_bytes(size_t es, int p, int N, int M) {
+    const int C = line_chunks(N, M), NF = p == 3 ? 4 : p, NU = p == 1 ? 2 : 4, NV = p == 1 ? 2 : (p == 2 ? 4 : 8);
+    return kTabHeader + es * (size_t)(8 + 2 * tab_round(p * p) + (2 * kEndRows + 3 * M) * NV + tab_round(C * M * NF) +
+                                      tab_round(C * M * NU) + 2 * tab_round(C * p * p) + 8);
 }
-// Chunk and interface types of the compact factor form: 0 = first, 1 = interior, 2 = last.
-__host__ __device__ inline int chunk_type(const Chunks& c, int k) { return k == 0 ? 0 : (k == c.C - 1 ? 2 : 1); }
-__host__ __device__ inline int iface_type(const Chunks& c, int k) { return k == 0 ? 0 : (k == c.C - 2 ? 2 : 1); }
-
-// Chunked LU of a banded 1-D operator A (half-bandwidth p), truncated-SPIKE form.
-//   lu[r][0..p-1]  multipliers: forward row r subtracts lu[r][i-1] * y[r-i]
-//   lu[r][p]       1 / U[r][r]
-//   lu[r][p+j]     U[r][r+j], j = 1..p
-//   spk[r][0..p-1] V (right spike of the chunk holding r), spk[r][p..2p-1] W (left spike)
-//   E[k][p][p]     (I - W_{k+1}^top V_k^bottom)^{-1} for the interface between chunks k and k+1
-// Every product is chunk-local: entries coupling two chunks are carried by the spikes.
-//
-// Compact form: with uniform open knots every interior chunk (1 .. C-2) of an operator
-// has bitwise identical factors, so three chunk types suffice whatever N is:
-//   luc[t][o][2p+1], spkc[t][o][2p] for o < mmax (= base + 2p), Ec[t][p][p], t in {0,1,2}.
-struct FactorV {
-    Chunks ch;
-    const void* lu;
-    const void* spk;
-    const void* E;
-    int compact;  // 1 if luc/spkc/Ec are valid (interior chunks verified identical)
-    int mmax;
-    const void* luc;
-    const void* spkc;
-    const void* Ec;
-    // the compact factors already in the padded shared-memory layout of the line kernels
-    // (fac_pad_elems elements; one bulk copy stages them), or NULL
-    const void* fpad;
+// One operator of a direction; band: its rows [N][2p+1] instead of factors (the explicit operator of
+// the middle y pass).
+struct TabJob {
+    const double *M, *K, *G;
+    double aM, aK, aG;
+    int N, chunk;
+    void* out;
+    int band;
+};
+struct TabJobs {
+    TabJob job[5];
+    int n;
+    void* mw;  // the slot's mean wind in the working precision (2 values)
+    double wind_x, wind_y;
+    double tol;  // products of transfers below it are dropped
+    int slots;   // slots written, sbytes apart (the same operators in each)
+    long long sbytes;
 };
 
 // ---- tables and factorisation (FP64, wf_tables.cu) ---------------------------------
@@ -99,16 +100,8 @@ cudaError_t launch_gauss(double* xi, double* w, int q, cudaStream_t s);
 cudaError_t launch_basis(const double* xi, int q, int n, int p, double L, double* B, double* D, cudaStream_t s);
 cudaError_t launch_assemble(const double* B, const double* D, const double* w, int q, int n, int p, double h,
                             double* Mb, double* Kb, double* Gb, cudaStream_t s);
-// A = aM M + aK K + aG G: full band (band64) and chunked factors; diag[0] = 1.0 if a pivot was
-// below 1e-300 ||A||_inf, diag[1] = largest neglected spike entry (truncation measure).
-cudaError_t launch_factor(const double* Mb, const double* Kb, const double* Gb, double aM, double aK, double aG,
-                          int N, int p, Chunks ch, double* band64, double* lu64, double* spk64, double* E64,
-                          double* work64, double* diag, cudaStream_t s);
-cudaError_t launch_to_f32(const double* src, float* dst, size_t n, cudaStream_t s);
-// Compact copies of chunk types 0/1/2 (see FactorV); diag[2] = 1.0 if an interior chunk differs
-// from chunk 1 bit for bit (then the compact form must not be used).
-cudaError_t launch_compact(const double* lu, const double* spk, const double* E, int p, Chunks ch, int mmax,
-                           double* luc, double* spkc, double* Ec, double* diag, cudaStream_t s);
+// every table of jobs.job[0 .. n-1], for jobs.slots slots
+cudaError_t launch_line_tables(int prec, int p, const TabJobs& jobs, cudaStream_t s);
 // out[r][e*q+a] = sum_l B[e][a][l] coef[r][e+l]  (1-D spline factor at Gauss points)
 cudaError_t launch_factor_points(int prec, const double* coef, int rank, int n, int p, const double* B,
                                  void* out, cudaStream_t s);
@@ -172,31 +165,33 @@ struct MmsArgs {
 cudaError_t launch_forcing(int prec, const MmsArgs& a, void* out, double s1, cudaStream_t s);
 cudaError_t launch_advance_time(double* t, double dt, cudaStream_t s);
 
-// ---- line solves (wf_solve.cu) -------------------------------------------
+// ---- line passes (wf_lines.cuh) -------------------------------------------------------
 struct LineArgs {
-    int G;       // lines per CTA of the compact-factor kernels (0: the launcher's rule; else an upper bound)
-    int rpw;     // x pass: lines per warp (0: as many as the chunks allow; 1, 2: at most that many)
+    int N, M, C, J;  // line length, chunk length and count; J: see the factor tables (largest of the slots)
+    int uni;     // every operator of the handle has uniform factors
+    int G;       // x pass: rows per CTA at most (0: the launcher's rule)
     int nlines;  // number of independent lines
     int pitch;   // row pitch of the fields (elements)
     int narr;    // 1 or 2 arrays (blockIdx.y)
     const void* in[2];
     void* out[2];
-    FactorV f[2];
-    const void* premul[2];  // y pass only: band applied along the line before the solve (or NULL)
-    double prescale[2];     // y pass only: factor of that band
-    const void* base[2];    // y pass only: out = base + solution (or NULL: out = solution)
-    int* status;            // y pass only: guard flag for out[0] (or NULL)
+    const void* tab[2];     // factor tables
+    const void* base[2];    // y pass: out = base + solution (or NULL: out = solution)
+    const void* band;       // middle y pass: rows of the explicit operator
+    int* status;            // y pass: guard flag for out[0] (or NULL)
     int* tstatus;           // x pass: flag word whose bit 4 records a bounded wait that gave up
-    int in_dead;            // y pass: the input arrays are dead after the pass (a kernel may use them
-                            // as scratch)
     long long wait_ns;      // limit of a bounded device wait (ns of %globaltimer; 0: give up at once)
     double tmax;
-    Batch b;  // per scenario: in, out, factors, premul, base, status
+    Batch b;  // per scenario: in, out, tab, base, band, status, tstatus
 };
-cudaError_t launch_xsolve(int prec, int p, const LineArgs& a, cudaStream_t s);
-cudaError_t launch_ysolve(int prec, int p, const LineArgs& a, cudaStream_t s);
-// compact-factor form (wf_linefast.cu); returns cudaErrorNotSupported when it cannot
-// take the arguments (factors not compact, more than 256 threads, shared memory)
+// kind 0: x pass; 1: y pass; 2: middle y pass of a Strang step (in: the x-solved right-hand side, base: T,
+// tab: M^y and Y_+, out: T**, a field of its own)
+cudaError_t launch_lines_p1_f32(int kind, const LineArgs& l, cudaStream_t s);
+cudaError_t launch_lines_p2_f32(int kind, const LineArgs& l, cudaStream_t s);
+cudaError_t launch_lines_p3_f32(int kind, const LineArgs& l, cudaStream_t s);
+cudaError_t launch_lines_p1_f64(int kind, const LineArgs& l, cudaStream_t s);
+cudaError_t launch_lines_p2_f64(int kind, const LineArgs& l, cudaStream_t s);
+cudaError_t launch_lines_p3_f64(int kind, const LineArgs& l, cudaStream_t s);
 // Raise (never lower) the dynamic shared memory a kernel may be launched with.  The limit is a
 // property of the kernel, read when a launch is made; the launches captured in a graph keep the
 // size each needed, so a later, smaller request for the same kernel (another pass, other launch
@@ -210,12 +205,6 @@ inline cudaError_t allow_dynamic_smem(K kern, size_t bytes) {
     return cudaFuncSetAttribute(reinterpret_cast<const void*>(kern), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)bytes);
 }
-cudaError_t launch_line_fast(int prec, int p, bool xdir, const LineArgs& a, cudaStream_t s);
-// elements of the padded factor block of one operator (chunk rows mmax), and the kernel that
-// writes it from the compact factors (luc, spkc, Ec in the working precision)
-size_t fac_pad_elems(int p, int mmax);
-cudaError_t launch_pad_factors(int prec, int p, int mmax, const void* luc, const void* spkc, const void* Ec,
-                               void* fpad, cudaStream_t s);
 
 // ---- persistent line passes (wf_persist.cu) -----------------------------------------
 // After the quadrature launch of a Peaceman-Rachford step (one F per step), one launch runs the
@@ -224,7 +213,6 @@ cudaError_t launch_pad_factors(int prec, int p, int mmax, const void* luc, const
 struct PersistHost {
     int prec, p;
     LineArgs x, y;            // two arrays each (R, Phi)
-    int xG, yG;               // x lines and y columns per tile (0: rule)
     int nslots_cap;           // slot capacity of the handle (counter blocks)
     long long wait_ns;
     int* status;              // slot-0 flag word
@@ -237,9 +225,10 @@ struct PersistHost {
 };
 struct PersistPlan {
     int nxg, nyg, narr, cstride, ctas;
-    size_t smem;
 };
-bool persist_supported(int prec, int p, int wind_rank);
+cudaError_t persist_p1(const PersistHost& h, PersistPlan* plan, bool launch, cudaStream_t s);
+cudaError_t persist_p2(const PersistHost& h, PersistPlan* plan, bool launch, cudaStream_t s);
+cudaError_t persist_p3(const PersistHost& h, PersistPlan* plan, bool launch, cudaStream_t s);
 // plan (and, with launch, enqueue: counter reset + one kernel) of one step; cudaErrorNotSupported
 // when the persistent form cannot take these arguments
 cudaError_t persist_step(const PersistHost& h, PersistPlan* plan, bool launch, cudaStream_t s);
@@ -247,9 +236,5 @@ cudaError_t persist_step(const PersistHost& h, PersistPlan* plan, bool launch, c
 // returns the count (entries past cap are not written) and the items of one slot
 int persist_items(const PersistPlan& plan, const int* slots, int nslots, int gs, int4* out, int cap,
                   int* items_per_slot);
-
-// launch-shape helpers shared with the host driver
-int line_rows_per_cta(int prec);
-size_t line_smem_bytes(int prec, const Chunks& ch);
 
 }  // namespace wf

@@ -1,0 +1,8 @@
+// Line passes of degree 1, FP64.
+#include "wf_lines_body.cuh"
+
+namespace wf {
+
+cudaError_t launch_lines_p1_f64(int kind, const LineArgs& l, cudaStream_t s) { return by_chunk<double, 1>(kind, l, s); }
+
+}  // namespace wf

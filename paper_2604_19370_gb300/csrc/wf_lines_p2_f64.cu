@@ -1,0 +1,8 @@
+// Line passes of degree 2, FP64.
+#include "wf_lines_body.cuh"
+
+namespace wf {
+
+cudaError_t launch_lines_p2_f64(int kind, const LineArgs& l, cudaStream_t s) { return by_chunk<double, 2>(kind, l, s); }
+
+}  // namespace wf

@@ -1,0 +1,8 @@
+// Line passes of degree 3, FP64.
+#include "wf_lines_body.cuh"
+
+namespace wf {
+
+cudaError_t launch_lines_p3_f64(int kind, const LineArgs& l, cudaStream_t s) { return by_chunk<double, 3>(kind, l, s); }
+
+}  // namespace wf

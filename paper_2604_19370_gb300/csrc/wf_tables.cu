@@ -3,9 +3,9 @@
 // Paper: the 1-D mass, stiffness and advection matrices of Sec. 3.1 ("Matrix
 // formulation") and the banded direct solvers of Sec. 4 ("Cost of directional
 // implicit solves").  Every directional operator is a combination
-// aM M + aK K + aG G of these matrices; its LU factors are computed here per
-// chunk of rows (truncated SPIKE partitioning, Polizzi & Sameh 2006) so that
-// the line solves of every step run with many independent chunks per line.
+// aM M + aK K + aG G of these matrices; its LU factors are computed here
+// together with the transfers of a recursion's state through chunks of rows, so
+// that the line solves of every step run with many chunks per line at once.
 #include <math.h>
 
 #include "wf_internal.h"
@@ -133,193 +133,324 @@ __global__ void k_assemble(const double* __restrict__ B, const double* __restric
     Gb[idx] = g;
 }
 
-__device__ inline void atomic_max_nonneg(double* addr, double v) {
-    // non-negative doubles order like their bit patterns
-    atomicMax(reinterpret_cast<unsigned long long*>(addr), (unsigned long long)__double_as_longlong(v));
-}
-
-// Chunk-local banded solve with the factors of one chunk (rows s .. s+m-1);
-// x has stride `stride` and holds the right-hand side on entry.
-__device__ void chunk_solve64(const double* lu, int s, int m, int p, double* x, int stride) {
-    const int W = 2 * p + 1;
-    for (int o = 0; o < m; ++o) {
-        const int r = s + o;
-        double v = x[(size_t)o * stride];
-        for (int i = 1; i <= p && o - i >= 0; ++i) v -= lu[(size_t)r * W + i - 1] * x[(size_t)(o - i) * stride];
-        x[(size_t)o * stride] = v;
+// Factor tables of one operator per block (layout: wf_internal.h).  A thread owns a chunk of rows and runs the
+// banded LU recursion (FP64, no pivoting) from the first row of the line down to its chunk, so every row has
+// the factors of one sequential elimination; one division a row.
+template <typename P, int PD>
+__global__ void __launch_bounds__(128) k_line_tables(const __grid_constant__ TabJobs jobs) {
+    constexpr int W = 2 * PD + 1, NF = PD == 3 ? 4 : PD, NU = PD == 1 ? 2 : 4, S = PD * PD;
+    const TabJob& jb = jobs.job[blockIdx.x];
+    const long long off = (long long)blockIdx.y * jobs.sbytes;
+    const int N = jb.N, M = jb.chunk, C = (N + M - 1) / M, tid = threadIdx.x;
+    char* out = static_cast<char*>(jb.out) + off;
+    auto entry = [&](int r, int d) {
+        const int col = r + d - PD;
+        const size_t o = (size_t)r * W + d;
+        return (col >= 0 && col < N) ? jb.aM * jb.M[o] + jb.aK * jb.K[o] + jb.aG * jb.G[o] : 0.0;
+    };
+    if (blockIdx.x == 0 && tid == 0) {
+        P* mw = reinterpret_cast<P*>(static_cast<char*>(jobs.mw) + off);
+        mw[0] = (P)jobs.wind_x;
+        mw[1] = (P)jobs.wind_y;
     }
-    for (int o = m - 1; o >= 0; --o) {
-        const int r = s + o;
-        double v = x[(size_t)o * stride];
-        for (int j = 1; j <= p && o + j < m; ++j) v -= lu[(size_t)r * W + p + j] * x[(size_t)(o + j) * stride];
-        x[(size_t)o * stride] = v * lu[(size_t)r * W + p];
+    if (jb.band) {
+        P* b = reinterpret_cast<P*>(out);
+        for (int i = tid; i < N * W; i += blockDim.x) b[i] = (P)entry(i / W, i % W);
+        return;
     }
-}
-
-// One thread per chunk: band of A, chunk-local LU without pivoting, and the spikes.
-__global__ void k_factor(const double* __restrict__ Mb, const double* __restrict__ Kb, const double* __restrict__ Gb,
-                         double aM, double aK, double aG, int N, int p, Chunks ch, double* band, double* lu,
-                         double* spk, double* work, double* diag) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= ch.C) return;
-    const int W = 2 * p + 1, S = 2 * p;
-    const int s = chunk_start(ch, k), m = chunk_len(ch, k), e = s + m;
-    double anorm = 0.0;
-    for (int r = s; r < e; ++r) {
-        double rs = 0.0;
-        for (int d = 0; d < W; ++d) {
-            const int col = r + d - p;
-            const size_t o = (size_t)r * W + d;
-            double v = (col >= 0 && col < N) ? aM * Mb[o] + aK * Kb[o] + aG * Gb[o] : 0.0;
-            band[o] = v;
-            work[o] = (col >= s && col < e) ? v : 0.0;
-            lu[o] = 0.0;
-            rs += fabs(v);
-        }
-        anorm = rs > anorm ? rs : anorm;
-        for (int c = 0; c < S; ++c) spk[(size_t)r * S + c] = 0.0;
-    }
-    // the norm must cover the whole matrix; chunk-local is a lower bound that is
-    // close to it for these operators (diagonally dominant bands of similar rows)
-    bool singular = false;
-    for (int r = s; r < e; ++r) {
-        double piv = work[(size_t)r * W + p];
-        if (!(fabs(piv) > 1e-300 * anorm)) {
-            singular = true;
-            piv = 1.0;
-        }
-        const double inv = 1.0 / piv;
-        for (int i = 1; i <= p && r + i < e; ++i) {
-            const size_t ri = (size_t)(r + i) * W;
-            const double l = work[ri + p - i] * inv;
-            lu[ri + i - 1] = l;
-            for (int j = 1; j <= p; ++j)
-                if (r + j < e) work[ri + p - i + j] -= l * work[(size_t)r * W + p + j];
-            work[ri + p - i] = 0.0;
-        }
-        lu[(size_t)r * W + p] = inv;
-        for (int j = 1; j <= p; ++j) lu[(size_t)r * W + p + j] = (r + j < e) ? work[(size_t)r * W + p + j] : 0.0;
-    }
-    if (singular) diag[0] = 1.0;
-    // right spike V = A_k^{-1} B_k (coupling to the first p unknowns of chunk k+1)
-    if (k + 1 < ch.C) {
-        for (int c = 0; c < p; ++c) {
-            double* x = spk + (size_t)s * S + c;
-            for (int o = 0; o < m; ++o) {
-                const int r = s + o, col = e + c, d = col - r + p;
-                x[(size_t)o * S] = (d >= 0 && d < W) ? band[(size_t)r * W + d] : 0.0;
+    constexpr int NV = PD == 1 ? 2 : (PD == 2 ? 4 : 8), D = 2 * PD, EW = 2 * kEndRows;
+    __shared__ int s_uni, s_J, s_bad, s_Ju;
+    __shared__ double s_l[PD], s_u[PD], s_inv, s_T[2][PD][PD];  // uniform factors and transfers
+    __shared__ double s_W[2 * D][EW];   // columns of B^{-1} at the first and last 2p unknowns, near each end
+    __shared__ double s_H[2 * D][4 * D];
+    if (tid == 0) s_uni = 0, s_J = 0, s_bad = 0, s_Ju = 0;
+    __syncthreads();
+    int* hdr = reinterpret_cast<int*>(out);
+    P* gl = reinterpret_cast<P*>(out + kTabHeader);
+    P* gu = gl + 4;
+    P* gT = gu + 4;
+    P* VT = gT + 2 * tab_round(S);
+    P* VB = VT + (kEndRows + M) * NV;
+    P* F = VB + (kEndRows + 2 * M) * NV;
+    P* U = F + tab_round(C * M * NF);
+    P* Pf = U + tab_round(C * M * NU);
+    P* Pb = Pf + tab_round(C * S);
+    for (int k = tid; k < C; k += blockDim.x) {
+        double u[PD][PD], inv[PD];  // rows r-1 .. r-p: u_{r-i,r-i+j} and 1 / u_{r-i,r-i}
+        double st[PD][PD];          // unit states carried through the chunk: [basis][value, nearest first]
+        for (int a = 0; a < PD; ++a) {
+            inv[a] = 0.0;
+            for (int b = 0; b < PD; ++b) {
+                u[a][b] = 0.0;
+                st[a][b] = a == b ? 1.0 : 0.0;
             }
-            chunk_solve64(lu, s, m, p, x, S);
         }
-    }
-    // left spike W = A_k^{-1} C_k (coupling to the last p unknowns of chunk k-1)
-    if (k > 0) {
-        for (int c = 0; c < p; ++c) {
-            double* x = spk + (size_t)s * S + p + c;
-            for (int o = 0; o < m; ++o) {
-                const int r = s + o, col = s - p + c, d = col - r + p;
-                x[(size_t)o * S] = (d >= 0 && d < W) ? band[(size_t)r * W + d] : 0.0;
+        double anorm = 0.0;
+        for (int r = 0; r < (k + 1) * M; ++r) {
+            double w[W], l[PD];
+            bool pad = r >= N;
+            double rs = 0.0;
+            for (int d = 0; d < W; ++d) {
+                w[d] = pad ? (d == PD ? 1.0 : 0.0) : entry(r, d);
+                rs += fabs(w[d]);
             }
-            chunk_solve64(lu, s, m, p, x, S);
-        }
-    }
-}
-
-// One thread per interface k (between chunks k and k+1): E_k = (I - W_{k+1}^top V_k^bottom)^{-1}
-// by Gauss-Jordan with partial pivoting, and the truncation measure (largest entry of
-// the spike blocks the truncated reduced system neglects).
-__global__ void k_interface(int p, Chunks ch, const double* __restrict__ spk, double* E, double* diag) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k + 1 >= ch.C) return;
-    const int S = 2 * p;
-    const int s0 = chunk_start(ch, k), m0 = chunk_len(ch, k);
-    const int s1 = chunk_start(ch, k + 1), m1 = chunk_len(ch, k + 1);
-    double A[kMaxP][2 * kMaxP];
-    for (int a = 0; a < p; ++a) {
-        for (int c = 0; c < p; ++c) {
-            double v = (a == c) ? 1.0 : 0.0;
-            for (int t = 0; t < p; ++t)
-                v -= spk[(size_t)(s1 + a) * S + p + t] * spk[(size_t)(s0 + m0 - p + t) * S + c];
-            A[a][c] = v;
-            A[a][p + c] = (a == c) ? 1.0 : 0.0;
-        }
-    }
-    for (int col = 0; col < p; ++col) {
-        int piv = col;
-        for (int r = col + 1; r < p; ++r)
-            if (fabs(A[r][col]) > fabs(A[piv][col])) piv = r;
-        if (piv != col)
-            for (int c = 0; c < 2 * p; ++c) {
-                double t = A[col][c];
-                A[col][c] = A[piv][c];
-                A[piv][c] = t;
+            if (!pad && rs > anorm) anorm = rs;
+#pragma unroll
+            for (int i = PD; i >= 1; --i) {
+                l[i - 1] = w[PD - i] * inv[i - 1];
+#pragma unroll
+                for (int j = 1; j <= PD; ++j) w[PD - i + j] -= l[i - 1] * u[i - 1][j - 1];
             }
-        double d = A[col][col];
-        if (!(fabs(d) > 1e-300)) {
-            diag[0] = 1.0;
-            d = 1.0;
+            double piv = w[PD];
+            if (!(fabs(piv) > 1e-300 * anorm)) {
+                s_bad = 1;
+                piv = 1.0;
+            }
+            const double iv = 1.0 / piv;
+            for (int a = PD - 1; a > 0; --a) {
+                inv[a] = inv[a - 1];
+                for (int b = 0; b < PD; ++b) u[a][b] = u[a - 1][b];
+            }
+            inv[0] = iv;
+            for (int b = 0; b < PD; ++b) u[0][b] = w[PD + 1 + b];
+            if (r >= k * M) {
+                for (int c = 0; c < NF; ++c) F[(size_t)r * NF + c] = c < PD ? (P)l[c < PD ? c : 0] : P(0);
+                U[(size_t)r * NU] = (P)iv;
+                for (int c = 1; c < NU; ++c) U[(size_t)r * NU + c] = c <= PD ? (P)(w[c <= PD ? PD + c : 0] * iv) : P(0);
+                for (int b = 0; b < PD; ++b) {
+                    double y = 0.0;
+                    for (int a = 0; a < PD; ++a) y -= l[a] * st[b][a];
+                    for (int a = PD - 1; a > 0; --a) st[b][a] = st[b][a - 1];
+                    st[b][0] = y;
+                }
+            }
         }
-        const double inv = 1.0 / d;
-        for (int c = 0; c < 2 * p; ++c) A[col][c] *= inv;
-        for (int r = 0; r < p; ++r) {
-            if (r == col) continue;
-            const double f = A[r][col];
-            for (int c = 0; c < 2 * p; ++c) A[r][c] -= f * A[col][c];
-        }
+        for (int a = 0; a < PD; ++a)
+            for (int b = 0; b < PD; ++b) Pf[(size_t)k * S + a * PD + b] = (P)st[b][a];
+        // backward: the chunk's own U rows from its last one up
+        for (int a = 0; a < PD; ++a)
+            for (int b = 0; b < PD; ++b) st[a][b] = a == b ? 1.0 : 0.0;
+        for (int r = (k + 1) * M - 1; r >= k * M; --r)
+            for (int b = 0; b < PD; ++b) {
+                double z = 0.0;
+                for (int a = 0; a < PD; ++a) z -= (double)U[(size_t)r * NU + 1 + a] * st[b][a];
+                for (int a = PD - 1; a > 0; --a) st[b][a] = st[b][a - 1];
+                st[b][0] = z;
+            }
+        for (int a = 0; a < PD; ++a)
+            for (int b = 0; b < PD; ++b) Pb[(size_t)k * S + a * PD + b] = (P)st[b][a];
     }
-    for (int a = 0; a < p; ++a)
-        for (int c = 0; c < p; ++c) E[(size_t)k * p * p + a * p + c] = A[a][p + c];
-    // The reduced system of interface k neglects the bottom of chunk k's left spike
-    // (zero for k = 0) and the top of chunk k+1's right spike (zero for k+1 = C-1).
-    double tr = 0.0;
-    for (int a = 0; a < p; ++a)
-        for (int c = 0; c < p; ++c) {
-            if (k > 0) tr = fmax(tr, fabs(spk[(size_t)(s0 + m0 - p + a) * S + p + c]));
-            if (k + 1 < ch.C - 1) tr = fmax(tr, fabs(spk[(size_t)(s1 + a) * S + c]));
+    __syncthreads();
+    // Uniform factors: the fixed point of the elimination of an interior row (row 2p), if it converges.
+    const double ulp = sizeof(P) == 4 ? 1e-12 : 4e-16;
+    if (tid == 0 && N > 4 * PD) {
+        double u[PD][PD], inv[PD], l[PD], w[W];
+        for (int a = 0; a < PD; ++a) {
+            inv[a] = 0.0;
+            for (int b = 0; b < PD; ++b) u[a][b] = 0.0;
         }
-    (void)m1;
-    atomic_max_nonneg(diag + 1, tr);
-}
-
-// Compact factors: chunk types 0 (first), 1 (interior, represented by chunk 1), 2 (last);
-// interface types 0 (k = 0), 1 (interior, interface 1), 2 (k = C-2).  One thread per
-// (row offset o < mmax); thread 0 also copies E and every thread checks interior
-// chunks against chunk 1.
-__global__ void k_compact(const double* __restrict__ lu, const double* __restrict__ spk, const double* __restrict__ E,
-                          int p, Chunks ch, int mmax, double* luc, double* spkc, double* Ec, double* diag) {
-    const int W = 2 * p + 1, S = 2 * p;
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o < mmax) {
-        const int src_chunk[3] = {0, ch.C >= 3 ? 1 : 0, ch.C - 1};
-        for (int t = 0; t < 3; ++t) {
-            const int k = src_chunk[t];
-            const bool ok = o < chunk_len(ch, k);
-            const size_t r = (size_t)chunk_start(ch, k) + o;
-            for (int d = 0; d < W; ++d) luc[((size_t)t * mmax + o) * W + d] = ok ? lu[r * W + d] : 0.0;
-            for (int c = 0; c < S; ++c) spkc[((size_t)t * mmax + o) * S + c] = ok ? spk[r * S + c] : 0.0;
+        int still = 0;
+        for (int it = 0; it < 4096 && still < PD + 2; ++it) {
+            for (int d = 0; d < W; ++d) w[d] = entry(2 * PD, d);
+            for (int i = PD; i >= 1; --i) {
+                l[i - 1] = w[PD - i] * inv[i - 1];
+                for (int j = 1; j <= PD; ++j) w[PD - i + j] -= l[i - 1] * u[i - 1][j - 1];
+            }
+            const double iv = 1.0 / w[PD];
+            bool same = fabs(iv - inv[0]) <= ulp * fabs(iv);
+            for (int b = 0; b < PD; ++b)
+                same = same && fabs(w[PD + 1 + b] - u[0][b]) <= ulp * fabs(w[PD]);
+            still = same ? still + 1 : 0;
+            for (int a = PD - 1; a > 0; --a) {
+                inv[a] = inv[a - 1];
+                for (int b = 0; b < PD; ++b) u[a][b] = u[a - 1][b];
+            }
+            inv[0] = iv;
+            for (int b = 0; b < PD; ++b) u[0][b] = w[PD + 1 + b];
         }
-        bool same = true;
-        for (int k = 2; k + 1 < ch.C && o < ch.base; ++k) {
-            const size_t r1 = (size_t)chunk_start(ch, 1) + o, rk = (size_t)chunk_start(ch, k) + o;
-            for (int d = 0; d < W; ++d) same &= lu[rk * W + d] == lu[r1 * W + d];
-            for (int c = 0; c < S; ++c) same &= spk[rk * S + c] == spk[r1 * S + c];
+        bool ok = still >= PD + 2 && isfinite(inv[0]);
+        // multipliers and rows as they will be stored, then the transfers through M rows and J
+        for (int a = 0; a < PD; ++a) {
+            s_l[a] = (double)(P)l[a];
+            s_u[a] = (double)(P)(u[0][a] * inv[0]);
         }
-        if (!same) diag[2] = 1.0;
+        s_inv = (double)(P)inv[0];
+        for (int dir = 0; dir < 2; ++dir) {
+            const double* c = dir ? s_u : s_l;
+            for (int b = 0; b < PD; ++b) {
+                double st[PD];
+                for (int a = 0; a < PD; ++a) st[a] = a == b ? 1.0 : 0.0;
+                for (int i = 0; i < M; ++i) {
+                    double y = 0.0;
+                    for (int a = 0; a < PD; ++a) y -= c[a] * st[a];
+                    for (int a = PD - 1; a > 0; --a) st[a] = st[a - 1];
+                    st[0] = y;
+                }
+                for (int a = 0; a < PD; ++a) s_T[dir][a][b] = st[a];
+            }
+            double prod[PD][PD], big = 1.0;
+            for (int a = 0; a < PD; ++a)
+                for (int b = 0; b < PD; ++b) prod[a][b] = a == b ? 1.0 : 0.0;
+            int J = 0;
+            while (ok && big > jobs.tol && (J + 1) * M <= kEndRows) {
+                double nx[PD][PD];
+                big = 0.0;
+                for (int a = 0; a < PD; ++a)
+                    for (int b = 0; b < PD; ++b) {
+                        nx[a][b] = 0.0;
+                        for (int q = 0; q < PD; ++q) nx[a][b] += prod[a][q] * s_T[dir][q][b];
+                        big = fmax(big, fabs(nx[a][b]));
+                    }
+                for (int a = 0; a < PD; ++a)
+                    for (int b = 0; b < PD; ++b) prod[a][b] = nx[a][b];
+                ++J;
+            }
+            ok = ok && big <= jobs.tol;
+            s_Ju = J > s_Ju ? J : s_Ju;
+        }
+        s_uni = ok ? 1 : 0;
     }
-    if (o == 0 && ch.C > 1) {
-        const int src_if[3] = {0, ch.C >= 4 ? 1 : 0, ch.C - 2};
-        for (int t = 0; t < 3; ++t)
-            for (int c = 0; c < p * p; ++c) Ec[t * p * p + c] = E[(size_t)src_if[t] * p * p + c];
-        bool same = true;
-        for (int k = 2; k < ch.C - 2; ++k)
-            for (int c = 0; c < p * p; ++c) same &= E[(size_t)k * p * p + c] == E[(size_t)p * p + c];
-        if (!same) diag[2] = 1.0;
+    __syncthreads();
+    const bool uni = s_uni != 0;
+    if (uni) {
+        // The ends: the system B has constant factors, E = A - B is nonzero in the first and last 2p x 2p
+        // blocks.  Rows 0 .. n1-1 and n - n2 .. of the line are kept (all of a short line, where both ends see
+        // each other); s_W[c]: column of B^{-1} at unknown c (c < 2p: the first ones, then the last ones).
+        const bool all = N <= EW;
+        const int len = all ? N : EW;  // rows of s_W: 0 .. len-1, for the last ones N - len .. N-1
+        if (tid < 2 * D) {
+            const bool bot = tid >= D;
+            double* w = s_W[tid];
+            const int at = bot ? len - 2 * D + tid : tid;
+            for (int i = 0; i < len; ++i) {
+                double y = i == at ? 1.0 : 0.0;
+                for (int a = 0; a < PD; ++a)
+                    if (i - 1 - a >= 0) y -= s_l[a] * w[i - 1 - a];
+                w[i] = y;
+            }
+            for (int i = len - 1; i >= 0; --i) {
+                double z = w[i] * s_inv;
+                for (int a = 0; a < PD; ++a)
+                    if (i + 1 + a < len) z -= s_u[a] * w[i + 1 + a];
+                w[i] = z;
+            }
+        }
+        __syncthreads();
+        if (tid == 0) {
+            // g = H z: H = (I + E W)^{-1} E over the end unknowns (first 2p, last 2p)
+            double E[2 * D][2 * D];
+            for (int a = 0; a < 2 * D; ++a)
+                for (int b = 0; b < 2 * D; ++b) {
+                    E[a][b] = 0.0;
+                    if ((a < D) != (b < D)) continue;
+                    const int i = a < D ? a : N - 2 * D + a, j = b < D ? b : N - 2 * D + b;
+                    const int d = j - i + PD;
+                    if (d < 0 || d >= W) continue;
+                    double lu = 0.0;  // (L U)_ij
+                    for (int m = (i > j ? i : j) - PD; m <= (i < j ? i : j); ++m) {
+                        if (m < 0) continue;
+                        const double lm = i == m ? 1.0 : s_l[i - m - 1];
+                        const double um = (j == m ? 1.0 : s_u[j - m - 1]) / s_inv;
+                        lu += lm * um;
+                    }
+                    E[a][b] = entry(i, d) - lu;
+                }
+            auto Wat = [&](int a, int c) {  // row of end unknown a, column of end unknown c
+                const bool ba = a >= D, bc = c >= D;
+                if (!all && ba != bc) return 0.0;
+                return s_W[c][ba ? len - 2 * D + a : a];
+            };
+            const int n = 2 * D;
+            for (int a = 0; a < n; ++a)
+                for (int b = 0; b < n; ++b) {
+                    double v = a == b ? 1.0 : 0.0;
+                    for (int q = 0; q < n; ++q) v += E[a][q] * Wat(q, b);
+                    s_H[a][b] = v;
+                    s_H[a][n + b] = E[a][b];
+                }
+            bool ok = true;
+            for (int col = 0; col < n; ++col) {
+                int pv = col;
+                for (int r = col + 1; r < n; ++r)
+                    if (fabs(s_H[r][col]) > fabs(s_H[pv][col])) pv = r;
+                ok = ok && fabs(s_H[pv][col]) > 1e-300;
+                for (int c = 0; c < 2 * n; ++c) {
+                    const double t = s_H[col][c];
+                    s_H[col][c] = s_H[pv][c];
+                    s_H[pv][c] = t;
+                }
+                const double iv = 1.0 / s_H[col][col];
+                for (int c = 0; c < 2 * n; ++c) s_H[col][c] *= iv;
+                for (int r = 0; r < n; ++r) {
+                    if (r == col) continue;
+                    const double f = s_H[r][col];
+                    for (int c = 0; c < 2 * n; ++c) s_H[r][c] -= f * s_H[col][c];
+                }
+            }
+            if (!ok) s_uni = 0;
+        }
+        __syncthreads();
+        const int J = s_Ju, kB = C - J - 1 > 0 ? C - J - 1 : 0, n = 2 * D;
+        for (int i = tid; i < (J < C ? J : C) * M; i += blockDim.x)
+            for (int c = 0; c < NV; ++c) {
+                double v = 0.0;
+                if (c < D && i < N)
+                    for (int a = 0; a < n; ++a)
+                        if (a < D || all) v += s_W[a][i] * s_H[a][n + c];
+                VT[(size_t)i * NV + c] = (P)v;
+            }
+        for (int i = tid; i < (C - kB) * M; i += blockDim.x) {
+            const int row = kB * M + i, o = row - (N - len);
+            for (int c = 0; c < NV; ++c) {
+                double v = 0.0;
+                if (c < D && row < N && o >= 0)
+                    for (int a = 0; a < n; ++a)
+                        if (a >= D || all) v += s_W[a][o] * s_H[a][n + D + c];
+                VB[(size_t)i * NV + c] = (P)v;
+            }
+        }
+        if (tid < 4) {
+            gl[tid] = tid < PD ? (P)s_l[tid < PD ? tid : 0] : P(0);
+            gu[tid] = tid == 0 ? (P)s_inv : (tid <= PD ? (P)s_u[tid - 1 < PD ? tid - 1 : 0] : P(0));
+        }
+        for (int i = tid; i < 2 * S; i += blockDim.x)
+            gT[(i / S) * tab_round(S) + i % S] = (P)s_T[i / S][(i % S) / PD][i % PD];
     }
-}
-
-__global__ void k_to_f32(const double* __restrict__ src, float* dst, size_t n) {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = (float)src[i];
+    __syncthreads();
+    // J: the smallest count of transfers whose product is below tol, for every chunk and direction (as
+    // many as there are chunks on that side where none is)
+    for (int q = tid; q < 2 * C; q += blockDim.x) {
+        const int k = q >> 1, step = (q & 1) ? 1 : -1;
+        const P* T = (q & 1) ? Pb : Pf;
+        double prod[PD][PD];
+        for (int a = 0; a < PD; ++a)
+            for (int b = 0; b < PD; ++b) prod[a][b] = a == b ? 1.0 : 0.0;
+        int J = 0;
+        for (int i = k + step; i >= 0 && i < C; i += step) {
+            // the state of chunk i counts as long as the transfers between it and chunk k do
+            double big = 0.0;
+            for (int a = 0; a < PD; ++a)
+                for (int b = 0; b < PD; ++b) big = fmax(big, fabs(prod[a][b]));
+            if (J > 0 && big <= jobs.tol) break;
+            ++J;
+            double nx[PD][PD];
+            for (int a = 0; a < PD; ++a)
+                for (int b = 0; b < PD; ++b) {
+                    nx[a][b] = 0.0;
+                    for (int c = 0; c < PD; ++c) nx[a][b] += prod[a][c] * (double)T[(size_t)i * S + c * PD + b];
+                }
+            for (int a = 0; a < PD; ++a)
+                for (int b = 0; b < PD; ++b) prod[a][b] = nx[a][b];
+        }
+        atomicMax(&s_J, J);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        hdr[0] = s_uni;
+        hdr[1] = s_Ju;
+        hdr[2] = s_J;
+        hdr[3] = s_bad;
+    }
 }
 
 template <typename P>
@@ -417,28 +548,15 @@ cudaError_t launch_assemble(const double* B, const double* D, const double* w, i
     return cudaGetLastError();
 }
 
-cudaError_t launch_factor(const double* Mb, const double* Kb, const double* Gb, double aM, double aK, double aG,
-                          int N, int p, Chunks ch, double* band64, double* lu64, double* spk64, double* E64,
-                          double* work64, double* diag, cudaStream_t s) {
-    k_factor<<<blocks(ch.C, 64), 64, 0, s>>>(Mb, Kb, Gb, aM, aK, aG, N, p, ch, band64, lu64, spk64, work64, diag);
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
-    if (ch.C > 1) {
-        k_interface<<<blocks(ch.C - 1, 64), 64, 0, s>>>(p, ch, spk64, E64, diag);
-        err = cudaGetLastError();
+cudaError_t launch_line_tables(int prec, int p, const TabJobs& jobs, cudaStream_t s) {
+    const dim3 grid(jobs.n, jobs.slots);
+    const bool f32 = prec == 0;
+    switch (p) {
+        case 1: f32 ? k_line_tables<float, 1><<<grid, 128, 0, s>>>(jobs) : k_line_tables<double, 1><<<grid, 128, 0, s>>>(jobs); break;
+        case 2: f32 ? k_line_tables<float, 2><<<grid, 128, 0, s>>>(jobs) : k_line_tables<double, 2><<<grid, 128, 0, s>>>(jobs); break;
+        case 3: f32 ? k_line_tables<float, 3><<<grid, 128, 0, s>>>(jobs) : k_line_tables<double, 3><<<grid, 128, 0, s>>>(jobs); break;
+        default: return cudaErrorInvalidValue;
     }
-    return err;
-}
-
-cudaError_t launch_compact(const double* lu, const double* spk, const double* E, int p, Chunks ch, int mmax,
-                           double* luc, double* spkc, double* Ec, double* diag, cudaStream_t s) {
-    k_compact<<<blocks(mmax, 64), 64, 0, s>>>(lu, spk, E, p, ch, mmax, luc, spkc, Ec, diag);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_to_f32(const double* src, float* dst, size_t n, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    k_to_f32<<<blocks(n, 256), 256, 0, s>>>(src, dst, n);
     return cudaGetLastError();
 }
 
