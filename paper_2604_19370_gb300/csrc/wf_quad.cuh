@@ -21,7 +21,7 @@
 // at the points, 33 + 24 + 21 to the test rows, 8 to finish a row: 222, against 345 multiply-adds
 // with basis tables.
 //
-// Schedule: one warp per work item, a strip of 32 element columns (lane L <-> element column
+// Two schedules.  Serial: one warp per work item, a strip of 32 element columns (lane L <-> element column
 // X0 - p + L, outputs from lane p on) walking down a segment of rows.  Registers hold sliding windows
 // of p rows: x components of the coefficient rows and x components of the unfinished test rows,
 // 2 p (p+1) values in all.  Neighbour coefficients are loaded directly (the second and third load of a
@@ -599,13 +599,13 @@ __device__ __forceinline__ void quad_strip(const QuadArgs<P>& a, int lane, int X
 }
 
 // Resident warps (one-warp CTAs) per SM the registers are budgeted for.
-template <typename P, int PD>
+template <int PD>
 struct QuadOcc {
-    static constexpr int value = sizeof(P) == 4 ? (PD <= 2 ? 24 : 16) : 8;
+    static constexpr int value = PD <= 2 ? 24 : 16;
 };
 
 template <typename P, int PD, int WR, bool XO>
-__global__ void __launch_bounds__(32, QuadOcc<P, PD>::value) k_quad(const __grid_constant__ QuadArgs<P> a) {
+__global__ void __launch_bounds__(32, QuadOcc<PD>::value) k_quad(const __grid_constant__ QuadArgs<P> a) {
     constexpr int NB = PD + 1;
     __shared__ P accg[NB * NB * 32];  // fuel sums of the unfinished rows: [row mod NB][x component][lane]
     extern __shared__ __align__(16) unsigned char wind_rows[];
@@ -615,6 +615,349 @@ __global__ void __launch_bounds__(32, QuadOcc<P, PD>::value) k_quad(const __grid
     const int X0 = strip * (32 - PD), Y0 = sg * a.h;
     P* wsm = reinterpret_cast<P*>(wind_rows);
     quad_strip<P, PD, WR, XO>(a, lane, X0, Y0, accg, wsm);
+}
+
+// Row-parallel form: a CTA of NW warps walks down a strip NW element rows a round, a row per warp; x components
+// of the coefficient rows and the loads of the element rows go through rings in shared memory, and each warp
+// finishes the output row of its element row (the same sums in the same order as the serial form: the same
+// bits).  A segment recomputes p element rows once per CTA instead of once per warp, a small domain has the
+// latency of one row instead of 1 + p of them, and the rows of a fire, two to three times as long, are spread over
+// the warps of a CTA.  FP64 always takes it: the pipe issues a warp's instruction in 16 cycles, a quarter
+// of that per scheduler, so the warp with the fire's rows was alone at the end (8 x 259^2 cubic: FP64
+// pipe 71% of the kernel's time, quadrature 1135 us; now 867 us; 66^2: 57 -> 30; 1026^2: 640 -> 626).
+// In FP32 the shared-memory traffic costs about a tenth more instructions: see the rule in run_quad.
+template <typename P, int PD, int NW>
+struct RowsSmem {
+    static constexpr int NB = PD + 1, RS = NW + PD;  // ring of rows
+    static constexpr bool kApart = sizeof(P) == 4;
+    P comps[RS][NB][32];      // x components of coefficient rows
+    P add[RS][NB * NB][32];   // loads of an element row: [test row][x component]
+    P fuel[RS][NB * NB][32];  // its fuel sums
+    // FP32: its reaction loads, added last as the serial form does; FP64, which has this form alone, adds them
+    // to the others at once (1026^2: step 688 us, 708 with the third array)
+    P react[kApart ? RS : 1][NB * NB][32];
+    int hot_c[RS], hot_e[RS]; // coefficient rows above T_ig, element rows with fuel sums
+};
+
+template <typename P, int PD, int WR, bool XO, int NW, typename SM>
+__device__ __forceinline__ void quad_rows(const QuadArgs<P>& a, int lane, int w, int X0, int Y0, SM& sm, P* wsm) {
+    using E = El<PD, P>;
+    constexpr int NB = PD + 1, Q = PD + 1, WRm = WR > 0 ? WR : 1, RS = NW + PD;
+    const ElK<P>& K = a.K;
+    const P* T0 = scene_ptr(a.T, a.b);
+    P* Phi0 = scene_ptr(a.Phi, a.b);
+    P* R0 = scene_ptr(a.R, a.b);
+    const P* mw = scene_ptr(a.mw, a.b);
+    const int ex = X0 - PD + lane;  // element column of this lane; also its DOF column
+    const bool ex_ok = ex >= 0 && ex < a.nx;
+    const bool out_col = lane >= PD && ex < a.Nx;
+    const bool xb = X0 < 2 * PD || X0 + 31 >= a.nx;  // the strip reaches the x boundary
+    const Ends<PD, P> xe(ex, a.nx);
+    const int rows = min(a.h, a.Ny - Y0);  // output rows of this item
+    const int e0 = Y0 - PD, ne = rows + PD;  // element rows e0 .. e0 + ne - 1
+
+    P fx[WRm][Q], fy[WRm][Q];
+    const P mwx = a.cwx * mw[0], mwy = XO ? P(0) : a.cwy * mw[1];
+    if constexpr (WR > 0) {
+        const P* fxq = scene_ptr(a.fxq, a.b);
+        const P* fyq = scene_ptr(a.fyq, a.b);
+        const P* gxq = scene_ptr(a.gxq, a.b);
+        const P* gyq = scene_ptr(a.gyq, a.b);
+#pragma unroll
+        for (int r = 0; r < WR; ++r)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const size_t o = (size_t)r * a.nx * Q + (size_t)(ex_ok ? ex : 0) * Q + q;
+                fx[r][q] = ex_ok ? a.cwx * fxq[o] : P(0);
+                fy[r][q] = ex_ok ? a.cwy * fyq[o] : P(0);
+            }
+        // [row][x, y][r][point]
+        for (int i = threadIdx.x; i < ne * WR * Q; i += 32 * NW) {
+            const int row = i / (WR * Q), rq = i - row * WR * Q, r = rq / Q, q = rq - r * Q;
+            const int ey = e0 + row;
+            const bool ok = ey >= 0 && ey < a.ny;
+            const size_t o = (size_t)r * a.ny * Q + (size_t)(ok ? ey : 0) * Q + q;
+            wsm[(row * 2 + 0) * WR * Q + rq] = ok ? gxq[o] : P(0);
+            wsm[(row * 2 + 1) * WR * Q + rq] = ok ? gyq[o] : P(0);
+        }
+    }
+    const int shift = min(max(ex, 0), a.nx - 1) - ex;
+    auto row_of = [&](const P* f, int r) {
+        return f + ((long long)min(max(r, 0), a.Ny - 1) * a.pitch + ex);
+    };
+    auto fetch = [&](const P* row, P (&x)[NB]) {
+        const P* c = row + shift;
+#pragma unroll
+        for (int k = 0; k < NB; ++k) x[k] = __ldg(c + k);
+    };
+    auto xcomps = [&](P (&x)[NB], P (&c)[NB]) {
+        if (PD > 1 && xb) xe.apply(x);
+        E::comps(x, c);
+    };
+    auto gather = [&](const P (&m)[NB]) {
+        P kx[NB];
+        E::scatter(m, kx, K);
+        if (xb) {
+            xe.transpose(kx);
+#pragma unroll
+            for (int k = 0; k < NB; ++k) kx[k] = ex_ok ? kx[k] : P(0);
+        }
+        P r = kx[0];
+#pragma unroll
+        for (int k = 1; k < NB; ++k) r += __shfl_up_sync(kFull, kx[k], k);
+        return r;
+    };
+    auto ycomps = [&](bool edge, int e, P (&x)[NB], P (&c)[NB]) {
+        if (__builtin_expect(edge, 0)) Ends<PD, P>(e, a.ny).apply(x);
+        E::comps(x, c);
+    };
+    auto yrows = [&](bool edge, int e, const P (&eta)[NB], P (&add)[NB]) {
+        E::scatter(eta, add, K);
+        if (__builtin_expect(edge, 0)) Ends<PD, P>(e, a.ny).transpose(add);
+    };
+    // x components of coefficient row e0 + c into its slot
+    auto put = [&](int slot, P (&x)[NB]) {
+        const bool h = __any_sync(kFull, larger(x[0], x[PD]) > a.T_ig_lo);
+        P c[NB];
+        xcomps(x, c);
+#pragma unroll
+        for (int j = 0; j < NB; ++j) sm.comps[slot][j][lane] = c[j];
+        if (lane == 0) sm.hot_c[slot] = h;
+    };
+    const P c_chi = held(a.c_chi), C_d = held(a.C_d);
+    P nxt[NB];
+    for (int c = w; c < RS; c += NW) {
+        fetch(row_of(T0, e0 + c), nxt);
+        put(c, nxt);
+    }
+    fetch(row_of(T0, e0 + RS + w), nxt);
+    if (w < PD && lane == 0) sm.hot_e[RS - 1 - w] = 0;
+    __syncthreads();
+    int si = w;  // slot of row i: i mod RS
+    for (int i0 = 0; i0 < ne; i0 += NW) {
+        const int i = i0 + w, ey = e0 + i;
+        const bool edge = ey < PD || ey >= a.ny - PD;
+        const bool in = i < ne && ey >= 0 && ey < a.ny;
+        P add[NB][NB];  // [test row][x component]
+        P tc[NB][NB];   // tensor components of the element: [y component][x component]
+        bool hot = false;
+        if (in) {
+            int sl[NB];
+#pragma unroll
+            for (int l = 0; l < NB; ++l) sl[l] = si + l < RS ? si + l : si + l - RS;
+#pragma unroll
+            for (int l = 0; l < NB; ++l) hot = hot || sm.hot_c[sl[l]];
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                P x[NB], c[NB];
+#pragma unroll
+                for (int l = 0; l < NB; ++l) x[l] = sm.comps[sl[l]][j][lane];
+                ycomps(edge, ey, x, c);
+#pragma unroll
+                for (int m = 0; m < NB; ++m) tc[m][j] = c[m];
+            }
+            P yv[Q][NB], yd[Q][NB];  // [y point][x component]: T and its y derivative
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                P c[NB], v[Q], d[Q];
+#pragma unroll
+                for (int m = 0; m < NB; ++m) c[m] = tc[m][j];
+                E::value(c, v, K);
+                E::deriv(c, d, K);
+#pragma unroll
+                for (int b = 0; b < Q; ++b) {
+                    yv[b][j] = v[b];
+                    yd[b][j] = d[b];
+                }
+            }
+            P mu[Q][NB], nu[Q][NB];  // x sums of the value and x-flux terms, of the y flux
+#pragma unroll
+            for (int b = 0; b < Q; ++b) {
+                P T[Q], Tx[Q], Ty[Q], s[Q], gx[Q], gy[Q];
+                E::value(yv[b], T, K);
+                E::deriv(yv[b], Tx, K);
+                E::value(yd[b], Ty, K);
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    const P T3 = (T[q] * T[q]) * T[q];
+                    P src = mad(T[q], mad(-a.c_rad, T3, -c_chi), a.K0);
+                    P bx = mwx, by = mwy;
+#pragma unroll
+                    for (int r = 0; r < WR; ++r) {
+                        bx = mad(fx[r][q], wsm[(i * 2 + 0) * WR * Q + r * Q + b], bx);
+                        by = mad(fy[r][q], wsm[(i * 2 + 1) * WR * Q + r * Q + b], by);
+                    }
+                    src = mad(bx, Tx[q], src);
+                    if (!XO || WR > 0) src = mad(by, Ty[q], src);
+                    s[q] = src;
+                    const P vx = mad(a.C_nld, T3, C_d), vy = XO ? a.C_nld * T3 : vx;
+                    gx[q] = vx * Tx[q];
+                    gy[q] = vy * Ty[q];
+                }
+                E::sums_flux(s, gx, mu[b], K, K.kx);
+                E::sums(gy, nu[b], K);
+            }
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                P s[Q], f[Q], eta[NB], t[NB];
+#pragma unroll
+                for (int b = 0; b < Q; ++b) {
+                    s[b] = mu[b][j];
+                    f[b] = nu[b][j];
+                }
+                E::sums_flux(s, f, eta, K, K.ky);
+                yrows(edge, ey, eta, t);
+#pragma unroll
+                for (int l = 0; l < NB; ++l) add[l][j] = t[l];
+            }
+        } else {
+#pragma unroll
+            for (int l = 0; l < NB; ++l)
+#pragma unroll
+                for (int j = 0; j < NB; ++j) add[l][j] = P(0);
+        }
+        if (__builtin_expect(hot, 0)) {
+            // reaction: E and E phi at the points, their loads
+            const P* phi0 = scene_ptr(a.phi, a.b);
+            P pv[Q][NB], yv[Q][NB];
+            {
+                P pw[NB][NB];
+#pragma unroll
+                for (int l = 0; l < NB; ++l) {
+                    P x[NB];
+                    fetch(row_of(phi0, ey + l), x);
+                    xcomps(x, pw[l]);
+                }
+#pragma unroll
+                for (int j = 0; j < NB; ++j) {
+                    P x[NB], c[NB], v[Q];
+#pragma unroll
+                    for (int l = 0; l < NB; ++l) x[l] = pw[l][j];
+                    ycomps(edge, ey, x, c);
+                    E::value(c, v, K);
+#pragma unroll
+                    for (int b = 0; b < Q; ++b) pv[b][j] = v[b];
+#pragma unroll
+                    for (int m = 0; m < NB; ++m) c[m] = tc[m][j];
+                    E::value(c, v, K);
+#pragma unroll
+                    for (int b = 0; b < Q; ++b) yv[b][j] = v[b];
+                }
+            }
+            P me[Q][NB], mp[Q][NB];
+#pragma unroll
+            for (int b = 0; b < Q; ++b) {
+                P T[Q], ph[Q], Ev[Q], Ep[Q];
+                E::value(yv[b], T, K);
+                E::value(pv[b], ph, K);
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    const bool burn = T[q] > a.T_ig && ph[q] > a.phi_min;
+                    const P e = burn ? T[q] * arrhenius(a.Ta_l2, a.T_a, T[q]) : P(0);
+                    Ep[q] = e * ph[q];
+                    Ev[q] = a.heat_by_fuel ? Ep[q] : e;
+                }
+                E::sums(Ev, me[b], K);
+                E::sums(Ep, mp[b], K);
+            }
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                P s[Q], eta[NB], t[NB];
+#pragma unroll
+                for (int b = 0; b < Q; ++b) s[b] = me[b][j];
+                E::sums(s, eta, K);
+                yrows(edge, ey, eta, t);
+#pragma unroll
+                for (int l = 0; l < NB; ++l) {
+                    if (SM::kApart) me[l][j] = t[l];  // (Q = NB)
+                    else add[l][j] = mad(a.K_ign, t[l], add[l][j]);
+                }
+                if (Phi0) {
+#pragma unroll
+                    for (int b = 0; b < Q; ++b) s[b] = mp[b][j];
+                    E::sums(s, eta, K);
+                    yrows(edge, ey, eta, t);
+#pragma unroll
+                    for (int l = 0; l < NB; ++l) mp[l][j] = t[l];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int l = 0; l < NB; ++l)
+#pragma unroll
+                for (int j = 0; j < NB; ++j) {
+                    if (SM::kApart) sm.react[si][l * NB + j][lane] = me[l][j];
+                    if (Phi0) sm.fuel[si][l * NB + j][lane] = mp[l][j];
+                }
+        } else {
+            __syncthreads();
+        }
+#pragma unroll
+        for (int l = 0; l < NB; ++l)
+#pragma unroll
+            for (int j = 0; j < NB; ++j) sm.add[si][l * NB + j][lane] = add[l][j];
+        if (lane == 0) sm.hot_e[si] = hot;
+        put(si, nxt);  // coefficient row i + RS
+        __syncthreads();
+        if (i0 + NW < ne) fetch(row_of(T0, ey + RS + NW), nxt);
+        if (i >= PD && i < ne) {
+            P m[NB];
+            int sl = si - PD < 0 ? si - PD + RS : si - PD;
+            int any = 0;
+#pragma unroll
+            for (int l = PD; l >= 0; --l) {
+#pragma unroll
+                for (int j = 0; j < NB; ++j) m[j] = l == PD ? sm.add[sl][l * NB + j][lane] : m[j] + sm.add[sl][l * NB + j][lane];
+                if (__builtin_expect(sm.hot_e[sl], 0)) {
+                    any = 1;
+                    if constexpr (SM::kApart)
+#pragma unroll
+                        for (int j = 0; j < NB; ++j) m[j] = mad(a.K_ign, sm.react[sl][l * NB + j][lane], m[j]);
+                }
+                sl = sl + 1 < RS ? sl + 1 : 0;
+            }
+            const P r = a.Rw * gather(m);
+            P f = P(0);
+            if (Phi0 && __builtin_expect(any, 0)) {
+#pragma unroll
+                for (int j = 0; j < NB; ++j) m[j] = P(0);
+                sl = si - PD < 0 ? si - PD + RS : si - PD;
+#pragma unroll
+                for (int l = PD; l >= 0; --l) {
+                    if (sm.hot_e[sl])
+#pragma unroll
+                        for (int j = 0; j < NB; ++j) m[j] += sm.fuel[sl][l * NB + j][lane];
+                    sl = sl + 1 < RS ? sl + 1 : 0;
+                }
+                f = a.fscale * gather(m);
+            }
+            if (out_col) {
+                const size_t o = (size_t)ey * a.pitch + ex;
+                R0[o] = r;
+                if (Phi0) Phi0[o] = f;
+            }
+        }
+        si = si + NW < RS ? si + NW : si + NW - RS;
+    }
+}
+
+constexpr int kRowWarps = 4;
+
+template <typename P, int PD>
+struct RowOcc {  // CTAs per SM
+    static constexpr int value = sizeof(P) == 4 ? (PD <= 2 ? 6 : 4) : 2;
+};
+
+template <typename P, int PD, int WR, bool XO, int NW>
+__global__ void __launch_bounds__(32 * NW, RowOcc<P, PD>::value) k_quad_rows(const __grid_constant__ QuadArgs<P> a) {
+    extern __shared__ __align__(16) unsigned char wind_rows[];
+    if (!scene_active(a.b)) return;
+    using SM = RowsSmem<P, PD, NW>;
+    SM& sm = *reinterpret_cast<SM*>(wind_rows);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int sg = blockIdx.x / a.ns, strip = a.s0 + (blockIdx.x - sg * a.ns);
+    quad_rows<P, PD, WR, XO, NW>(a, lane, w, strip * (32 - PD), sg * a.h, sm,
+                                 reinterpret_cast<P*>(wind_rows + sizeof(SM)));
 }
 
 template <typename P>
@@ -690,27 +1033,6 @@ cudaError_t run_quad(const RhsArgs& r, cudaStream_t s) {
     a.nstrips = (r.Nx + (32 - PD) - 1) / (32 - PD);
     int sms = 152, dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // Segment height: a segment recomputes p element rows, so high ones do less work; but below about the
-    // resident number of warps per SM the SMs idle on latency.  The largest power of two from 64 down
-    // that gives nine tenths of the resident warps an item, then equal segments.  1026^2 FP32 step:
-    // 40.1 us at height 8 (its rule), 41.0 at 24, 46.1 at 32, 51.4 at 2; FP64: 764 at 32 (its rule), 802
-    // at 16; 66^2 FP64: 130 at 1 (its rule), 175 at 4; 4099^2 cubic: 702 at 64, 762 at 16.
-    int hgt = 64;
-    const long want = (long)QuadOcc<P, PD>::value * sms * 9 / 10;
-    while (hgt > 1 && (long)a.nstrips * ((r.Ny + hgt - 1) / hgt) * r.b.S < want) hgt /= 2;
-    if (r.seg > 0) hgt = r.seg;
-    if (hgt > r.Ny) hgt = r.Ny;
-    // the segment's wind factors stay within 48 KB of shared memory, beside the fuel sums
-    auto wind_bytes = [](int h) { return (size_t)2 * WR * (PD + 1) * (h + PD) * sizeof(P); };
-    while (hgt > 1 && wind_bytes(hgt) > 48 * 1024) hgt /= 2;
-    const int nseg = (r.Ny + hgt - 1) / hgt;
-    a.h = (r.Ny + nseg - 1) / nseg;
-    const size_t smem = wind_bytes(a.h);
-    auto kern = k_quad<P, PD, WR, XO>;
-    if (smem > 24 * 1024) {
-        cudaError_t e = allow_dynamic_smem(kern, smem);
-        if (e != cudaSuccess) return e;
-    }
     // interior strips: X0 >= 2p and X0 + 31 < nx
     int lo = (2 * PD + (32 - PD) - 1) / (32 - PD), hi = r.nx > 31 ? (r.nx - 32) / (32 - PD) + 1 : 0;
     if (lo > a.nstrips) lo = a.nstrips;
@@ -719,16 +1041,72 @@ cudaError_t run_quad(const RhsArgs& r, cudaStream_t s) {
     // the strips right of them in launches of their own (FP32 with interior strips)
     const bool parts = r.parts && sizeof(P) == 4 && hi > lo;
     const int cut[4] = {0, parts ? lo : a.nstrips, parts ? hi : a.nstrips, a.nstrips};
-    for (int k = 0; k < 3; ++k) {
-        a.s0 = cut[k];
-        a.ns = cut[k + 1] - cut[k];
-        if (a.ns <= 0) continue;
-        kern<<<dim3((unsigned)(a.ns * nseg), 1, r.b.S), 32, smem, s>>>(a);
-        count_launches(1);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+    // the segment's wind factors stay within 48 KB of shared memory, beside the sums
+    auto wind_bytes = [](int h) { return (size_t)2 * WR * (PD + 1) * (h + PD) * sizeof(P); };
+    const long strips = (long)a.nstrips * r.b.S;
+    auto launch = [&](auto kern, int hgt, int threads, size_t ring) {
+        if (r.seg > 0) hgt = r.seg;
+        if (hgt > r.Ny) hgt = r.Ny;
+        while (hgt > 1 && wind_bytes(hgt) > 48 * 1024) hgt /= 2;
+        const int nseg = (r.Ny + hgt - 1) / hgt;
+        a.h = threads == 32 ? (r.Ny + nseg - 1) / nseg : hgt;
+        const size_t smem = ring + wind_bytes(a.h);
+        if (smem > 24 * 1024) {
+            cudaError_t e = allow_dynamic_smem(kern, smem);
+            if (e != cudaSuccess) return e;
+        }
+        for (int k = 0; k < 3; ++k) {
+            a.s0 = cut[k];
+            a.ns = cut[k + 1] - cut[k];
+            if (a.ns <= 0) continue;
+            kern<<<dim3((unsigned)(a.ns * nseg), 1, r.b.S), threads, smem, s>>>(a);
+            count_launches(1);
+            cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    };
+    constexpr int NW = kRowWarps;
+    const size_t ring = sizeof(RowsSmem<P, PD, NW>);
+    if constexpr (sizeof(P) == 8) {
+        // Height by the FP64 pipe: rounds of NW element rows on the busiest SM, fewest first, then the lower
+        // segment (8 x 259^2 cubic, step at height 65 (its rule): 951 us, 1107 at 52, 982 at 33).
+        int h = r.Ny;
+        long best = 0;
+        for (int n = 1; n <= r.Ny && strips * (n - 1) < 8L * sms; ++n) {
+            const int hn = (r.Ny + n - 1) / n;
+            const long ctas = strips * ((r.Ny + hn - 1) / hn);
+            const long cost = (ctas + sms - 1) / sms * ((hn + PD + NW - 1) / NW);
+            if (best == 0 || cost <= best) best = cost, h = hn;
+        }
+        return launch(k_quad_rows<P, PD, WR, XO, NW>, h, 32 * NW, ring);
+    } else {
+        const double rows_sm = (double)strips * r.Ny / sms;  // element rows per SM
+        // Row-parallel while the rows are few enough for latency to decide; its height weighs the rounds of a
+        // segment against the element rows recomputed (a round is one row's latency; eight rows per SM take
+        // about as long to issue).  Step, serial / row-parallel: 130^2 16.4 / 13.9 us, 402^2 25.4 / 24.1
+        // (37 rows per SM), 642^2 26.7 / 28.5 (93); cubic 100 x 64 Strang 53 / 37, 515^2 46.9 / 37.2 (61), 643^2
+        // 47.7 / 42.0 (97), 803^2 50.5 / 52.3 (148); linear within 0.8 us up to 60.
+        if (rows_sm <= (PD <= 2 ? 48 : 128)) {
+            int h = NW - PD;
+            double best = 1e30;
+            for (int g = 1; g <= 16; ++g) {
+                const int hn = NW * g - PD;
+                const double cost = g + 0.125 * rows_sm * (hn + PD) / hn;
+                if (hn >= 1 && cost < best) best = cost, h = hn;
+            }
+            return launch(k_quad_rows<P, PD, WR, XO, NW>, h, 32 * NW, ring);
+        }
+        // Segment height of the serial form: a segment recomputes p element rows, so high ones do less work;
+        // but below about the resident number of warps per SM the SMs idle on latency.  The largest power of two
+        // from 64 down that gives nine tenths of the resident warps an item, then equal segments.
+        // 1026^2: 40.1 us at height 8 (its rule), 41.0 at 24, 46.1 at 32, 51.4 at 2; 4099^2
+        // cubic: 702 at 64 (its rule), 762 at 16.
+        int h = 64;
+        const long want = (long)QuadOcc<PD>::value * sms * 9 / 10;
+        while (h > 1 && strips * ((r.Ny + h - 1) / h) < want) h /= 2;
+        return launch(k_quad<P, PD, WR, XO>, h, 32, 0);
     }
-    return cudaSuccess;
 }
 
 // instantiations by wind rank (ranks 3 and 4 run as 4, rank 1 as 2: the unused factors are zero) and

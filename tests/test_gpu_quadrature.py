@@ -58,3 +58,31 @@ def test_quadrature_sizes_against_oracle(wf, nx, ny, p, prec):
     P = Problem(nx, ny, p, Lx, Ly, 1e-3, wind, fac, Params(scale_heat_by_fuel=bool(k % 2)), scheme, "ads")
     To, po = P.run(T0, f0, 2)
     assert_parity(T, phi, To, po, prec, rel_bar=1e-10 if prec == "fp64" else 1e-5)
+
+
+@pytest.mark.parametrize("nx,ny", [(5, 31), (29, 30), (64, 33), (91, 8)])
+@pytest.mark.parametrize("p", [1, 2, 3])
+@pytest.mark.parametrize("scheme", ["pr", "strang"])
+def test_serial_and_row_parallel_quadrature_agree(wf, nx, ny, p, scheme):
+    """FP32: a batch of more than 128 element rows per SM takes the serial form, one domain the row-parallel one;
+    a slot's bits are those of the domain alone."""
+    Lx, Ly, T0, f0, wind, fac = _case(nx, ny, p, 900 + nx + p, 2)
+    factors = np.concatenate([a.ravel() for a in fac])
+    prm = wf.wf_params_default(Lx=Lx, Ly=Ly, wind_x=wind[0], wind_y=wind[1], precision=wf.WF_FP32,
+                               scheme=wf.WF_PR if scheme == "pr" else wf.WF_STRANG_CN)
+    strips = -(-(nx + p) // (32 - p))
+    S = 130 * 152 // (strips * (ny + p)) + 1
+    with wf.Batch(nx, ny, p, 1e-3, prm, capacity=S) as b:
+        b.set_slot(S - 1, T0, f0, wind, 2, factors)
+        b.activate(S - 1)
+        b.step(2)
+        assert not b.status().any()
+        T, phi = b.state(S - 1)
+    sim = wf.Simulation(nx, ny, p, 1e-3, prm)
+    sim.set_state(T0, f0)
+    sim.set_wind(2, factors)
+    sim.step(2)
+    assert sim.sync() == wf.WF_OK
+    Ts, ps = sim.state()
+    sim.close()
+    assert np.array_equal(T, Ts) and np.array_equal(phi, ps)
