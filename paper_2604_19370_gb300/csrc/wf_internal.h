@@ -35,12 +35,6 @@ struct Batch {
     const int* budget;  // [S] step budgets (negative: unlimited) or nullptr (none)
 };
 #ifdef __CUDACC__
-template <typename T>
-__device__ __forceinline__ T* scene_ptr(T* p, const Batch& b) {
-    return p ? reinterpret_cast<T*>(reinterpret_cast<char*>(const_cast<typename std::remove_const<T>::type*>(p)) +
-                                    (long long)blockIdx.z * b.sbytes)
-             : p;
-}
 __device__ __forceinline__ bool scene_active(const Batch& b) {
     return (!b.active || b.active[blockIdx.z] != 0) && (!b.budget || b.budget[blockIdx.z] != 0);
 }
@@ -205,6 +199,37 @@ inline cudaError_t allow_dynamic_smem(K kern, size_t bytes) {
     return cudaFuncSetAttribute(reinterpret_cast<const void*>(kern), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)bytes);
 }
+
+// A launch that may begin while the last CTAs of the kernel before it in the stream drain (programmatic dependent
+// launch; the kernel begins with grid_wait): the launch latency and the start of the CTAs overlap that tail.
+template <typename... KA, typename... A>
+inline cudaError_t launch_overlapped(void (*kern)(KA...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                                     A... args) {
+    cudaLaunchConfig_t c = {};
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, KA(args)...);
+}
+#ifdef __CUDACC__
+// First statement of such a kernel: waits until the kernel before it is complete and its writes are visible.
+// `off` is added to every address the kernel reads, and passes through the wait, so that no load (a read-only one
+// neither) can be moved above it.  A grid of at most kEarlyCtas CTAs then lets the next kernel's CTAs start
+// beside it; larger ones leave that to their end, where the next kernel's CTAs no longer take room from theirs.  us per
+// step, no overlap / at the end / always early: 130^2 13.9 / 13.0 / 12.9, 100 x 64 cubic Strang 37.7 / 36.7 /
+// 35.2, 1026^2 34.8 / 33.9 / 35.6, 8 x 515^2 cubic 105.3 / 104.3 / 107.5.
+constexpr unsigned kEarlyCtas = 2 * 152;
+__device__ __forceinline__ void grid_wait(long long& off) {
+    asm volatile("griddepcontrol.wait;" : "+l"(off)::"memory");
+    if (gridDim.x * gridDim.y * gridDim.z <= kEarlyCtas) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
 
 // ---- persistent line passes (wf_persist.cu) -----------------------------------------
 // After the quadrature launch of a Peaceman-Rachford step (one F per step), one launch runs the

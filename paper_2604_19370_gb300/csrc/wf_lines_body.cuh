@@ -18,27 +18,31 @@ template <typename P, int PD, int M, bool UNI, int NT, bool STAGED>
 __global__ void __launch_bounds__(NT, NT > 512 ? 1 : LineOcc<P, M>::ctas) k_xlines(const __grid_constant__ PassArgs<P> a,
                                                                                    int nt) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    long long off = (long long)blockIdx.z * a.b.sbytes;
+    grid_wait(off);
     if (!scene_active(a.b)) return;
-    x_any<P, PD, M, UNI, STAGED>(a, (long long)blockIdx.z * a.b.sbytes, blockIdx.y, blockIdx.x, smem_raw, threadIdx.x, nt);
+    x_any<P, PD, M, UNI, STAGED>(a, off, blockIdx.y, blockIdx.x, smem_raw, threadIdx.x, nt);
 }
 
 template <typename P, int PD, int M, bool UNI, int NT>
 __global__ void __launch_bounds__(NT, NT > 512 ? 1 : LineOcc<P, M>::ctas) k_ylines(const __grid_constant__ PassArgs<P> a,
                                                                                    int ntiles) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    if (!scene_active(a.b)) return;
+    long long off = (long long)blockIdx.z * a.b.sbytes;
     const int cg = blockIdx.x / ntiles;
-    y_any<P, PD, M, UNI, false>(a, (long long)blockIdx.z * a.b.sbytes, blockIdx.y, cg, blockIdx.x - cg * ntiles, smem_raw,
-                                threadIdx.x);
+    grid_wait(off);
+    if (!scene_active(a.b)) return;
+    y_any<P, PD, M, UNI, false>(a, off, blockIdx.y, cg, blockIdx.x - cg * ntiles, smem_raw, threadIdx.x);
 }
 
 template <typename P, int PD, int M, bool UNI>
 __global__ void __launch_bounds__(512, 1) k_ymid(const __grid_constant__ PassArgs<P> a, const P* band, int ntiles) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    if (!scene_active(a.b)) return;
+    long long off = (long long)blockIdx.z * a.b.sbytes;
     const int cg = blockIdx.x / ntiles;
-    y_mid_any<P, PD, M, UNI>(a, band, (long long)blockIdx.z * a.b.sbytes, cg, blockIdx.x - cg * ntiles, smem_raw,
-                             threadIdx.x);
+    grid_wait(off);
+    if (!scene_active(a.b)) return;
+    y_mid_any<P, PD, M, UNI>(a, band, off, cg, blockIdx.x - cg * ntiles, smem_raw, threadIdx.x);
 }
 
 template <typename K, typename... A>
@@ -47,9 +51,9 @@ cudaError_t go(K kern, dim3 grid, int threads, size_t smem, cudaStream_t s, A...
         cudaError_t e = allow_dynamic_smem(kern, smem);
         if (e != cudaSuccess) return e;
     }
-    kern<<<grid, threads, smem, s>>>(args...);
-    count_launches(1);
-    return cudaGetLastError();
+    const cudaError_t e = launch_overlapped(kern, grid, threads, smem, s, args...);
+    if (e == cudaSuccess) count_launches(1);
+    return e;
 }
 
 template <typename P, int PD, int M, bool UNI>

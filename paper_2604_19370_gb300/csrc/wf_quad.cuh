@@ -290,17 +290,22 @@ struct QuadArgs {
     Batch b;
 };
 
+template <typename T>
+__device__ __forceinline__ T* at_slot(T* p, long long off) {
+    return p ? reinterpret_cast<T*>((char*)p + off) : p;
+}
+
 // One item: the strip at X0, rows [Y0, Y0 + h).  Rows and columns outside the domain are read at the
 // nearest one inside: the elements that use them lie outside themselves and contribute zero.
 template <typename P, int PD, int WR, bool XO>
-__device__ __forceinline__ void quad_strip(const QuadArgs<P>& a, int lane, int X0, int Y0, P* accg, P* wsm) {
+__device__ __forceinline__ void quad_strip(const QuadArgs<P>& a, long long off, int lane, int X0, int Y0, P* accg, P* wsm) {
     using E = El<PD, P>;
     constexpr int NB = PD + 1, Q = PD + 1, WRm = WR > 0 ? WR : 1;
     const ElK<P>& K = a.K;
-    const P* T0 = scene_ptr(a.T, a.b);
-    P* Phi0 = scene_ptr(a.Phi, a.b);
-    P* R0 = scene_ptr(a.R, a.b);
-    const P* mw = scene_ptr(a.mw, a.b);
+    const P* T0 = at_slot(a.T, off);
+    P* Phi0 = at_slot(a.Phi, off);
+    P* R0 = at_slot(a.R, off);
+    const P* mw = at_slot(a.mw, off);
     const int ex = X0 - PD + lane;  // element column of this lane; also its DOF column
     const bool ex_ok = ex >= 0 && ex < a.nx;
     const bool out_col = lane >= PD && ex < a.Nx;
@@ -313,10 +318,10 @@ __device__ __forceinline__ void quad_strip(const QuadArgs<P>& a, int lane, int X
     P fx[WRm][Q], fy[WRm][Q];
     const P mwx = a.cwx * mw[0], mwy = XO ? P(0) : a.cwy * mw[1];
     if constexpr (WR > 0) {
-        const P* fxq = scene_ptr(a.fxq, a.b);
-        const P* fyq = scene_ptr(a.fyq, a.b);
-        const P* gxq = scene_ptr(a.gxq, a.b);
-        const P* gyq = scene_ptr(a.gyq, a.b);
+        const P* fxq = at_slot(a.fxq, off);
+        const P* fyq = at_slot(a.fyq, off);
+        const P* gxq = at_slot(a.gxq, off);
+        const P* gyq = at_slot(a.gyq, off);
 #pragma unroll
         for (int r = 0; r < WR; ++r)
 #pragma unroll
@@ -509,7 +514,7 @@ __device__ __forceinline__ void quad_strip(const QuadArgs<P>& a, int lane, int X
             to_rows([&](const P(&eta)[NB], P(&add)[NB]) { E::scatter(eta, add, K); });
         if (__builtin_expect(hot > 0, 0)) {
             // reaction: E and E phi at the points, their loads into R and into the fuel sums
-            const P* phi0 = scene_ptr(a.phi, a.b);
+            const P* phi0 = at_slot(a.phi, off);
             P pv[Q][NB];
             {
                 P pw[NB][NB];
@@ -609,12 +614,14 @@ __global__ void __launch_bounds__(32, QuadOcc<PD>::value) k_quad(const __grid_co
     constexpr int NB = PD + 1;
     __shared__ P accg[NB * NB * 32];  // fuel sums of the unfinished rows: [row mod NB][x component][lane]
     extern __shared__ __align__(16) unsigned char wind_rows[];
+    long long off = (long long)blockIdx.z * a.b.sbytes;
+    grid_wait(off);
     if (!scene_active(a.b)) return;
     const int lane = threadIdx.x;
     const int sg = blockIdx.x / a.ns, strip = a.s0 + (blockIdx.x - sg * a.ns);
     const int X0 = strip * (32 - PD), Y0 = sg * a.h;
     P* wsm = reinterpret_cast<P*>(wind_rows);
-    quad_strip<P, PD, WR, XO>(a, lane, X0, Y0, accg, wsm);
+    quad_strip<P, PD, WR, XO>(a, off, lane, X0, Y0, accg, wsm);
 }
 
 // Row-parallel form: a CTA of NW warps walks down a strip NW element rows a round, a row per warp; x components
@@ -640,14 +647,14 @@ struct RowsSmem {
 };
 
 template <typename P, int PD, int WR, bool XO, int NW, typename SM>
-__device__ __forceinline__ void quad_rows(const QuadArgs<P>& a, int lane, int w, int X0, int Y0, SM& sm, P* wsm) {
+__device__ __forceinline__ void quad_rows(const QuadArgs<P>& a, long long off, int lane, int w, int X0, int Y0, SM& sm, P* wsm) {
     using E = El<PD, P>;
     constexpr int NB = PD + 1, Q = PD + 1, WRm = WR > 0 ? WR : 1, RS = NW + PD;
     const ElK<P>& K = a.K;
-    const P* T0 = scene_ptr(a.T, a.b);
-    P* Phi0 = scene_ptr(a.Phi, a.b);
-    P* R0 = scene_ptr(a.R, a.b);
-    const P* mw = scene_ptr(a.mw, a.b);
+    const P* T0 = at_slot(a.T, off);
+    P* Phi0 = at_slot(a.Phi, off);
+    P* R0 = at_slot(a.R, off);
+    const P* mw = at_slot(a.mw, off);
     const int ex = X0 - PD + lane;  // element column of this lane; also its DOF column
     const bool ex_ok = ex >= 0 && ex < a.nx;
     const bool out_col = lane >= PD && ex < a.Nx;
@@ -659,10 +666,10 @@ __device__ __forceinline__ void quad_rows(const QuadArgs<P>& a, int lane, int w,
     P fx[WRm][Q], fy[WRm][Q];
     const P mwx = a.cwx * mw[0], mwy = XO ? P(0) : a.cwy * mw[1];
     if constexpr (WR > 0) {
-        const P* fxq = scene_ptr(a.fxq, a.b);
-        const P* fyq = scene_ptr(a.fyq, a.b);
-        const P* gxq = scene_ptr(a.gxq, a.b);
-        const P* gyq = scene_ptr(a.gyq, a.b);
+        const P* fxq = at_slot(a.fxq, off);
+        const P* fyq = at_slot(a.fyq, off);
+        const P* gxq = at_slot(a.gxq, off);
+        const P* gyq = at_slot(a.gyq, off);
 #pragma unroll
         for (int r = 0; r < WR; ++r)
 #pragma unroll
@@ -818,7 +825,7 @@ __device__ __forceinline__ void quad_rows(const QuadArgs<P>& a, int lane, int w,
         }
         if (__builtin_expect(hot, 0)) {
             // reaction: E and E phi at the points, their loads
-            const P* phi0 = scene_ptr(a.phi, a.b);
+            const P* phi0 = at_slot(a.phi, off);
             P pv[Q][NB], yv[Q][NB];
             {
                 P pw[NB][NB];
@@ -951,12 +958,14 @@ struct RowOcc {  // CTAs per SM
 template <typename P, int PD, int WR, bool XO, int NW>
 __global__ void __launch_bounds__(32 * NW, RowOcc<P, PD>::value) k_quad_rows(const __grid_constant__ QuadArgs<P> a) {
     extern __shared__ __align__(16) unsigned char wind_rows[];
+    long long off = (long long)blockIdx.z * a.b.sbytes;
+    grid_wait(off);
     if (!scene_active(a.b)) return;
     using SM = RowsSmem<P, PD, NW>;
     SM& sm = *reinterpret_cast<SM*>(wind_rows);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int sg = blockIdx.x / a.ns, strip = a.s0 + (blockIdx.x - sg * a.ns);
-    quad_rows<P, PD, WR, XO, NW>(a, lane, w, strip * (32 - PD), sg * a.h, sm,
+    quad_rows<P, PD, WR, XO, NW>(a, off, lane, w, strip * (32 - PD), sg * a.h, sm,
                                  reinterpret_cast<P*>(wind_rows + sizeof(SM)));
 }
 
@@ -1059,10 +1068,10 @@ cudaError_t run_quad(const RhsArgs& r, cudaStream_t s) {
             a.s0 = cut[k];
             a.ns = cut[k + 1] - cut[k];
             if (a.ns <= 0) continue;
-            kern<<<dim3((unsigned)(a.ns * nseg), 1, r.b.S), threads, smem, s>>>(a);
-            count_launches(1);
-            cudaError_t e = cudaGetLastError();
+            const cudaError_t e =
+                launch_overlapped(kern, dim3((unsigned)(a.ns * nseg), 1, r.b.S), threads, smem, s, a);
             if (e != cudaSuccess) return e;
+            count_launches(1);
         }
         return cudaSuccess;
     };
