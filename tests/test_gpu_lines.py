@@ -73,6 +73,13 @@ def test_slow_decay_against_oracle(wf, Nx, Ny, p, scheme):
     _check(wf, Nx, Ny, p, "fp64", scheme, wind=(0.0, 0.0), kappa=3e6, hot=400.0, steps=1)
 
 
+@pytest.mark.parametrize("Nx,Ny", [(4, 17003), (17003, 4)])
+@pytest.mark.parametrize("scheme", ["pr", "strang"])
+def test_slow_decay_on_longest_lines_against_oracle(wf, Nx, Ny, scheme):
+    """More than 512 chunks whose states reach over several tiles."""
+    _check(wf, Nx, Ny, 2, "fp64", scheme, wind=(0.0, 0.0), kappa=3e6, hot=400.0, steps=1)
+
+
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
 @pytest.mark.parametrize("scheme", ["pr", "strang"])
 def test_slow_decay_beside_other_slots(wf, prec, scheme):
