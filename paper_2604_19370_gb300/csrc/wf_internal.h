@@ -62,6 +62,11 @@ struct Phys {
 //   Pf[C][p][p], Pb[C][p][p]  transfers through every chunk
 // every part rounded up to a multiple of four elements.
 constexpr int kTabHeader = 64;
+// FP32 takes uniform factors where an operator has them.  FP64 reads every row's factors: its pipe bounds the
+// passes, loads are free beside it, and the end corrections are a tenth to a half more multiply-adds (step, uniform /
+// table: 66^2 quadratic 51.4 / 47.5 us, 8 x 259^2 cubic 890 / 873, 1026^2 690 / 686).
+template <typename P>
+constexpr bool kUniformFactors = sizeof(P) == 4;
 constexpr int kEndRows = 128;  // J * M at most for the uniform form
 __host__ __device__ constexpr int tab_round(int n) { return (n + 3) & ~3; }
 inline int line_chunks(int N, int M) { return (N + M - 1) / M; }

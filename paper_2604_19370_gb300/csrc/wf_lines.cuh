@@ -698,7 +698,9 @@ __device__ __forceinline__ bool uniform_table(const void* tab, long long off) {
 template <typename P, int PD, int M, bool UNI, bool STAGED>
 __device__ __forceinline__ void x_any(const PassArgs<P>& a, long long off, int arr, int tile, unsigned char* smem, int tid,
                                       int nt) {
-    if (UNI || uniform_table(arr ? a.tab[1] : a.tab[0], off))
+    if constexpr (!kUniformFactors<P>)
+        x_tile<P, PD, M, false, STAGED>(a, off, arr, tile, smem, tid, nt);
+    else if (UNI || uniform_table(arr ? a.tab[1] : a.tab[0], off))
         x_tile<P, PD, M, true, STAGED>(a, off, arr, tile, smem, tid, nt);
     else
         x_tile<P, PD, M, false, STAGED>(a, off, arr, tile, smem, tid, nt);
@@ -706,7 +708,9 @@ __device__ __forceinline__ void x_any(const PassArgs<P>& a, long long off, int a
 template <typename P, int PD, int M, bool UNI, bool CG>
 __device__ __forceinline__ void y_any(const PassArgs<P>& a, long long off, int arr, int cg, int tile, unsigned char* smem,
                                       int tid) {
-    if (UNI || uniform_table(arr ? a.tab[1] : a.tab[0], off))
+    if constexpr (!kUniformFactors<P>)
+        y_tile<P, PD, M, false, CG>(a, off, arr, cg, tile, smem, tid);
+    else if (UNI || uniform_table(arr ? a.tab[1] : a.tab[0], off))
         y_tile<P, PD, M, true, CG>(a, off, arr, cg, tile, smem, tid);
     else
         y_tile<P, PD, M, false, CG>(a, off, arr, cg, tile, smem, tid);
@@ -714,7 +718,9 @@ __device__ __forceinline__ void y_any(const PassArgs<P>& a, long long off, int a
 template <typename P, int PD, int M, bool UNI>
 __device__ __forceinline__ void y_mid_any(const PassArgs<P>& a, const P* band, long long off, int cg, int tile,
                                           unsigned char* smem, int tid) {
-    if (UNI || (uniform_table(a.tab[0], off) && uniform_table(a.tab[1], off)))
+    if constexpr (!kUniformFactors<P>)
+        y_mid_tile<P, PD, M, false>(a, band, off, cg, tile, smem, tid);
+    else if (UNI || (uniform_table(a.tab[0], off) && uniform_table(a.tab[1], off)))
         y_mid_tile<P, PD, M, true>(a, band, off, cg, tile, smem, tid);
     else
         y_mid_tile<P, PD, M, false>(a, band, off, cg, tile, smem, tid);

@@ -128,7 +128,9 @@ cudaError_t run_kind(int kind, const LineArgs& l, cudaStream_t s) {
 
 template <typename P, int PD, int M>
 cudaError_t run_pass(int kind, const LineArgs& l, cudaStream_t s) {
-    return l.uni ? run_kind<P, PD, M, true>(kind, l, s) : run_kind<P, PD, M, false>(kind, l, s);
+    if constexpr (kUniformFactors<P>)
+        if (l.uni) return run_kind<P, PD, M, true>(kind, l, s);
+    return run_kind<P, PD, M, false>(kind, l, s);
 }
 
 template <typename P, int PD>

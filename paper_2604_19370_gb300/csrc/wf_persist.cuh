@@ -197,8 +197,7 @@ cudaError_t persist_prec(const PersistHost& h, PersistPlan* plan, bool launch, c
     if (h.prec == WF_FP32)
         return h.x.uni ? persist_by_chunk<float, PD, true>(h, plan, launch, s)
                        : persist_by_chunk<float, PD, false>(h, plan, launch, s);
-    return h.x.uni ? persist_by_chunk<double, PD, true>(h, plan, launch, s)
-                   : persist_by_chunk<double, PD, false>(h, plan, launch, s);
+    return persist_by_chunk<double, PD, false>(h, plan, launch, s);
 }
 
 }  // namespace

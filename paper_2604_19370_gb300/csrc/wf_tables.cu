@@ -242,8 +242,9 @@ __global__ void __launch_bounds__(128) k_line_tables(const __grid_constant__ Tab
     }
     __syncthreads();
     // Uniform factors: the fixed point of the elimination of an interior row (row 2p), if it converges.
-    const double ulp = sizeof(P) == 4 ? 1e-12 : 4e-16;
-    if (tid == 0 && N > 4 * PD) {
+    // (FP32: kUniformFactors, wf_internal.h)
+    const double ulp = 1e-12;
+    if (kUniformFactors<P> && tid == 0 && N > 4 * PD) {
         double u[PD][PD], inv[PD], l[PD], w[W];
         for (int a = 0; a < PD; ++a) {
             inv[a] = 0.0;
