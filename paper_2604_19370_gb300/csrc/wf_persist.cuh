@@ -85,8 +85,14 @@ __device__ __forceinline__ void slot_done(const PersistArgs<P>& A, int* cnt, int
     }
 }
 
-template <typename P, int PD, int M, bool UNI>
-__global__ void __launch_bounds__(512, 1) k_lines_persist(const __grid_constant__ PersistArgs<P> A) {
+// CTAs per SM the registers are budgeted for, by the CTA's threads.
+template <typename P, int M, int NT>
+struct PersistOcc {
+    static constexpr int ctas = (sizeof(P) == 4 ? (M <= 17 ? 1536 : 1024) : 512) / NT;
+};
+
+template <typename P, int PD, int M, bool UNI, int NT>
+__global__ void __launch_bounds__(NT, PersistOcc<P, M, NT>::ctas) k_lines_persist(const __grid_constant__ PersistArgs<P> A) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_item, s_go;
     const int tid = threadIdx.x;
@@ -130,7 +136,7 @@ __global__ void __launch_bounds__(512, 1) k_lines_persist(const __grid_constant_
     }
 }
 
-template <typename P, int PD, int M, bool UNI>
+template <typename P, int PD, int M, bool UNI, int NT>
 cudaError_t persist_typed(const PersistHost& h, PersistPlan* plan, bool launch, cudaStream_t s) {
     PersistArgs<P> A;
     memset(&A, 0, sizeof(A));
@@ -138,8 +144,8 @@ cudaError_t persist_typed(const PersistHost& h, PersistPlan* plan, bool launch, 
     pass_args(h.y, h.y.N, A.y);
     int ntx = 0, nty = 0;
     size_t sx = 0, sy = 0;
-    if (!x_geometry<P, PD, M>(h.x, 512, 72 * 1024, A.x, &ntx, &sx) ||
-        !y_geometry<P, PD, M>(h.y, 512, A.y, &nty, &sy) || !A.x.staged)
+    if (!x_geometry<P, PD, M>(h.x, NT, 72 * 1024, A.x, &ntx, &sx) ||
+        !y_geometry<P, PD, M>(h.y, NT, A.y, &nty, &sy) || !A.x.staged)
         return cudaErrorNotSupported;
     A.x.bulk = 0;
     A.sbytes = h.x.b.sbytes;
@@ -148,7 +154,7 @@ cudaError_t persist_typed(const PersistHost& h, PersistPlan* plan, bool launch, 
     A.nty = (A.y.C + A.y.KO - 1) / A.y.KO;
     const size_t smem = std::max(sx, sy);
     const int threads = std::max(ntx, nty);
-    auto kern = k_lines_persist<P, PD, M, UNI>;
+    auto kern = k_lines_persist<P, PD, M, UNI, NT>;
     cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0, sms = 152, dev = 0;
@@ -182,12 +188,21 @@ cudaError_t persist_typed(const PersistHost& h, PersistPlan* plan, bool launch, 
     return cudaGetLastError();
 }
 
+// CTAs of 256 threads where they hold both kinds of tile: an x tile uses at most that many (128 on 258 values),
+// so larger CTAs idle in the x pass (256 scenarios of
+// 258^2, step: 1175 us with 512 threads, 671 with 256; one 1026^2 domain 73).
+template <typename P, int PD, int M, bool UNI>
+cudaError_t persist_threads(const PersistHost& h, PersistPlan* plan, bool launch, cudaStream_t s) {
+    const cudaError_t e = persist_typed<P, PD, M, UNI, 256>(h, plan, launch, s);
+    return e == cudaErrorNotSupported ? persist_typed<P, PD, M, UNI, 512>(h, plan, launch, s) : e;
+}
+
 template <typename P, int PD, bool UNI>
 cudaError_t persist_by_chunk(const PersistHost& h, PersistPlan* plan, bool launch, cudaStream_t s) {
     switch (h.x.M) {
-        case 9: return persist_typed<P, PD, 9, UNI>(h, plan, launch, s);
-        case 17: return persist_typed<P, PD, 17, UNI>(h, plan, launch, s);
-        case 33: return persist_typed<P, PD, 33, UNI>(h, plan, launch, s);
+        case 9: return persist_threads<P, PD, 9, UNI>(h, plan, launch, s);
+        case 17: return persist_threads<P, PD, 17, UNI>(h, plan, launch, s);
+        case 33: return persist_threads<P, PD, 33, UNI>(h, plan, launch, s);
     }
     return cudaErrorNotSupported;
 }
