@@ -50,7 +50,7 @@ extern "C" {
 #define WF_EUNSTABLE (-4)    /* a temperature became non-finite or exceeded 1e5 K */
 #define WF_ETIMEOUT (-5)     /* a bounded device wait gave up */
 #define WF_ECUDA (-6)        /* a CUDA runtime call failed (no device, launch error, ...) */
-#define WF_ETRUNC (-7)       /* the chunked line solve could not reach its truncation tolerance */
+#define WF_ETRUNC (-7)       /* a line operator reaches too far for the handle (wf_set_mean_wind) */
 #define WF_ENOTFOUND (-8)    /* unknown request ticket */
 
 /* ---- choices ----------------------------------------------------------- */
@@ -203,12 +203,13 @@ int wf_kernel_times(wf_handle* h, double* ms, int* counts, char (*names)[48], in
  * Change the mean wind b (m/s) of a slot between steps (slot 0 for a handle of
  * wf_create), keeping its state: the runs of Sec. 7 change the wind direction
  * part-way (the Gran Canaria run: a south-westerly, then a westerly wind).  The
- * slot's implicit operators and their chunked factors are rebuilt on the GPU
+ * slot's implicit operators and their factor tables are rebuilt on the GPU
  * (FP64); the call waits for the handle's stream first.  Captured step graphs
- * stay valid (they address the factors, not their values).
- * Errors: WF_EINVAL, WF_ESINGULAR / WF_ETRUNC (the new operators cannot be
- * factored with the chunk length chosen at creation; the slot keeps its
- * previous wind), WF_ECUDA.
+ * stay valid (they address the factors, not their values); the handle captures
+ * its own again where the new operators reach over more chunks of a line.
+ * Errors: WF_EINVAL, WF_ESINGULAR / WF_ETRUNC (the inverse of a new operator
+ * decays far more slowly along a line than those of creation; the slot keeps
+ * its previous wind), WF_ECUDA.
  */
 int wf_set_mean_wind(wf_handle* h, int slot, double wind_x, double wind_y);
 
@@ -269,10 +270,10 @@ int wf_launch_count(unsigned long long* n);
  *             that one group's quadrature runs beside the other group's line
  *             passes; the groups join at the end of each wf_step call (and
  *             of each captured graph of steps).  Batches of two or more
- *             slots without manufactured forcing; profiled steps and
- *             wf_step_noalloc run the launches of form 1;
+ *             slots without manufactured forcing; profiled steps run the
+ *             launches of form 1, wf_step_noalloc those of form 0;
  *   shape[7]  slots per group of the persistent step's work order (the order
- *             keeps about six groups' fields live, sized for the L2 cache);
+ *             keeps about two groups' fields live, sized for the L2 cache);
  * 0 selects the built-in rule.
  * Every value changes the schedule only: every step form performs the same
  * operations in the same order, so the results are the same bits.  wf_autotune tunes one value at a

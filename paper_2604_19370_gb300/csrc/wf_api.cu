@@ -530,8 +530,8 @@ cudaError_t rhs_and_forcing(wf_handle* h, const RhsArgs& r) {
 cudaError_t enqueue_step_body(wf_handle* h);
 
 // The persistent form (one quadrature launch, then one launch over every line pass of every active
-// slot) takes PR with one F per step; tuning value 6 picks it (2) or the per-pass launches (1,
-// and the rule 0: measured faster on the ensemble and on a single domain).
+// slot) takes PR with one F per step; tuning value 6 picks it (2) or the per-pass launches (the rule:
+// measured faster on the ensemble and on a single domain).
 bool use_persist(const wf_handle* h) {
     // (a launch over a group of slots, gn > 0, takes the per-pass form: the persistent plan lists
     // every active slot of the handle)

@@ -1,6 +1,6 @@
 // Line solves of the directional operators (Sec. 4, "Cost of directional implicit solves": independent
-// banded 1-D systems along x or y), device code shared by the per-pass kernels (wf_lines.cu) and the
-// persistent one (wf_persist.cu).
+// banded 1-D systems along x or y), device code shared by the per-pass kernels (wf_lines_body.cuh) and the
+// persistent one (wf_persist.cuh).
 //
 // A line of N values is cut into C chunks of M; one thread owns one chunk of one line and keeps its M values in
 // registers from load to store.  The operator's LU factors are those of the whole line (wf_tables.cu).
@@ -22,7 +22,8 @@
 // are kept for J chunks from either end.  Every chunk then runs its recursions with factors in registers;
 // reading each row's factors from a table in the chunks near the ends made those the slowest of their CTA
 // (256 scenarios of 258^2, FP32: x pass 66, y pass 93 us).  Operators whose factors do not converge, whose
-// states reach further than kEndRows rows, and lines of less than 4p + 1 values take the table of exact factors.
+// states reach further than kEndRows rows, lines of less than 4p + 1 values, and FP64 (kUniformFactors) take the table
+// of exact factors.
 //
 // Against a chunk-local LU with spike corrections (three sweeps over shared memory, about 50 warp
 // instructions a value) this is about 9 multiply-adds a value from registers, and the chunk's loads are all

@@ -1109,8 +1109,8 @@ cudaError_t run_quad(const RhsArgs& r, cudaStream_t s) {
         // Segment height of the serial form: a segment recomputes p element rows, so high ones do less work;
         // but below about the resident number of warps per SM the SMs idle on latency.  The largest power of two
         // from 64 down that gives nine tenths of the resident warps an item, then equal segments.
-        // 1026^2: 40.1 us at height 8 (its rule), 41.0 at 24, 46.1 at 32, 51.4 at 2; 4099^2
-        // cubic: 702 at 64 (its rule), 762 at 16.
+        // Step, 1026^2: 34.7 us at height 8 (its rule), 34.5 at 13, 36.6 at 20, 38.9 at 30; 8 x 515^2
+        // cubic: 102.9 at 31 (its rule), 109 at 24, 118 at 52; 4099^2 cubic: 537 at 64 (its rule), 554 at 32, 550 at 128.
         int h = 64;
         const long want = (long)QuadOcc<PD>::value * sms * 9 / 10;
         while (h > 1 && strips * ((r.Ny + h - 1) / h) < want) h /= 2;

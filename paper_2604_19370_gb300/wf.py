@@ -339,9 +339,9 @@ TUNING_NAMES = ("x_lines_per_cta", "y_lines_per_cta", "quadrature_segment_rows",
 
 
 def wf_get_tuning(h) -> Tuple[int, ...]:
-    """(x lines per CTA, y lines per CTA, quadrature segment rows, x lines per warp, second-x-pass
-    lines per CTA, second-x-pass right-hand side (1 fused, 2 separate matvec), step form (1 per-pass
-    launches, 2 persistent), slots per group of the persistent order)."""
+    """(rows per x CTA, unused, quadrature segment rows, unused, rows per CTA of the second x pass, unused,
+    step form (0 the rule: a launch per pass, 1 a launch per pass and array, 2 persistent, 3 two slot
+    groups), slots per group of the persistent order)."""
     out = (ctypes.c_int * 8)()
     _check(lib().wf_get_tuning(h, out), "wf_get_tuning")
     return tuple(int(v) for v in out)
