@@ -132,6 +132,8 @@ struct wf_handle {
     int* p_cnt = nullptr;
     size_t p_items_cap = 0, p_cnt_cap = 0;
     bool p_dirty = true;
+    bool any_wind = false;  // launches that stay valid for every mean wind the handle accepts (the caller's graphs):
+                            // the kernels that ask each table for its form, tiles with the largest reach
     bool noalloc_run = false;  // wf_step_noalloc in progress: per-pass launches only
     void *T = nullptr, *phi = nullptr, *Phi = nullptr, *R = nullptr, *W = nullptr;
     int* status = nullptr;
@@ -460,6 +462,11 @@ LineArgs line_args(wf_handle* h, int xsite) {
     a.C = line_chunks(a.N, a.M);
     a.uni = h->uni ? 1 : 0;
     a.J = h->uni ? h->J[1] : std::max(h->J[0], h->J[1]);
+    if (h->any_wind) {
+        const int most = h->reach_most[xdir ? 0 : 1];
+        a.uni = 0;
+        a.J = most == INT_MAX ? a.C : std::min(a.C, most / a.M + 1);
+    }
     a.nlines = xdir ? h->Ny : h->Nx;
     a.G = xsite == 1 ? h->tune[0] : (xsite == 2 ? h->tune[4] : 0);
     a.pitch = h->pitch;
@@ -1763,9 +1770,12 @@ extern "C" int wf_step_noalloc(wf_handle* h, void* T, void* fuel, int pitch, int
     h->W = scratch + 2 * kNoallocMaxElems;
     h->pitch = pitch;
     cudaError_t e = cudaSuccess;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess) (void)cudaGetLastError();
+    h->any_wind = cs == cudaStreamCaptureStatusActive;
     h->noalloc_run = true;  // the persistent step's buffers may not exist yet: per-pass launches
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k) e = enqueue_step(h);
-    h->noalloc_run = false;
+    h->noalloc_run = h->any_wind = false;
     h->T = save[0];
     h->phi = save[1];
     h->Phi = save[2];

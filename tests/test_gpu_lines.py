@@ -103,3 +103,36 @@ def test_slow_decay_beside_other_slots(wf, prec, scheme):
     Ts, ps = sim.state()
     sim.close()
     assert np.array_equal(T, Ts) and np.array_equal(phi, ps)
+
+
+@pytest.mark.parametrize("n", [60, 300])
+def test_captured_steps_follow_a_new_wind(wf, n):
+    """A caller's graph of allocation-free steps addresses the factors: replayed after a change to a wind whose
+    operators reach further, it gives the bits of steps launched then."""
+    torch = pytest.importorskip("torch")
+    Lx, Ly, T0, f0 = _state(n, n, 2, 900.0)
+    prm = wf.wf_params_default(Lx=Lx, Ly=Ly, wind_x=0.5, wind_y=-0.5, precision=wf.WF_FP32)
+    sim = wf.Simulation(n, n, 2, 1e-3, prm)
+    st = torch.cuda.Stream()
+    wf.wf_set_stream(sim.h, st.cuda_stream)
+    a = [torch.tensor(x, dtype=torch.float32, device="cuda") for x in (T0, f0)]
+    step = lambda: wf.wf_step_noalloc(sim.h, a[0].data_ptr(), a[1].data_ptr(), n + 2, 2)  # noqa: E731
+    with torch.cuda.stream(st):
+        assert step() == wf.WF_OK  # looks the scratch address up before the capture
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        assert step() == wf.WF_OK
+    wf.wf_set_mean_wind(sim.h, 1500.0, -1200.0)
+    out = []
+    for run in (g.replay, step):
+        for x, x0 in zip(a, (T0, f0)):
+            x.copy_(torch.tensor(x0, dtype=torch.float32))
+        torch.cuda.synchronize()
+        with torch.cuda.stream(st):
+            run()
+        torch.cuda.synchronize()
+        out.append([x.cpu().numpy().copy() for x in a])
+    sim.close()
+    assert np.isfinite(out[1][0]).all()
+    assert all(np.array_equal(x, y) for x, y in zip(*out))
