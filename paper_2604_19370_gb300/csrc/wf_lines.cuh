@@ -396,7 +396,7 @@ struct PassArgs {
     // shared memory; y: G columns and CK chunks per CTA, of which those of its tile of KO are written
     int G, sp, CK, KO, halo;
     int cells;  // x: states of a CTA in values / p
-    int staged, bulk;  // x: rows go through shared memory; by bulk copies
+    int staged, bulk;  // x: rows go through shared memory; by bulk copies of row_values values
     const P* in[2];
     P* out[2];
     const P* base[2];
@@ -414,6 +414,14 @@ __device__ __forceinline__ T* shift(T* p, long long off) {
              : p;
 }
 
+// Values of a row in shared memory: its N values up to a multiple of 16 bytes, whatever the row pitch of the field (a
+// caller of the allocation-free step chooses that).  Bulk copies move as many: rows of a multiple of 16 bytes have them.
+template <typename P>
+__host__ __device__ __forceinline__ int row_values(int N) {
+    constexpr int per = 16 / (int)sizeof(P);
+    return (N + per - 1) / per * per;
+}
+
 // ---- x tile: G rows of one array, the whole CTA (G * chunks threads, the chunks rounded up to whole
 // warps) -----------------------------------------------------------------------------------
 // shared memory: [16] mbarrier, [G][sp] rows (staged), [chunks][G][p] states, [4p][G] end values
@@ -426,7 +434,7 @@ __device__ __forceinline__ void x_tile(const PassArgs<P>& a, long long off, int 
     const void* tab = shift(one ? a.tab[1] : a.tab[0], off);
     const int N = a.N, C = a.C, G = a.G, L = 32 / G;
     const int j0 = tile * G, rows = min(G, a.nlines - j0);
-    const size_t row_bytes = (size_t)a.pitch * sizeof(P);
+    const size_t row_bytes = (size_t)row_values<P>(N) * sizeof(P);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem);
     P* rowbuf = reinterpret_cast<P*>(smem + 16);
     P* st = rowbuf + (STAGED ? (size_t)G * a.sp : 0);
@@ -743,7 +751,7 @@ bool x_geometry(const LineArgs& l, int max_threads, size_t smem_budget, PassArgs
         const int L = 32 / G, slots = sizeof(P) == 4 ? 32 : 16;
         // shared-memory row stride: the rows of a warp start L banks apart (chunk lengths are odd), so its
         // lanes hit distinct banks; 16-byte multiple for bulk copies
-        int sp = l.pitch;
+        int sp = row_values<P>(l.N);
         if (L < slots)
             while (sp % (2 * L) != L || (sp * sizeof(P)) % 16 != 0) ++sp;
         else

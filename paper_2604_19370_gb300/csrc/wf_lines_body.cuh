@@ -86,6 +86,8 @@ cudaError_t run_x(const LineArgs& l, cudaStream_t s) {
                             : go(k_xlines<P, PD, M, UNI, 1024, false>, grid, nt, smem, s, a, nt);
         if (!a.staged) return go(k_xlines<P, PD, M, UNI, 512, false>, grid, nt, smem, s, a, nt);
     }
+    // (shorter chunks mean rows of at most 1600 values, which always fit: there is no other kernel for them)
+    if (!a.staged) return cudaErrorInvalidValue;
     return go(k_xlines<P, PD, M, UNI, 512, true>, grid, nt, smem, s, a, nt);
 }
 
