@@ -322,7 +322,8 @@ int wf_batch_create(int nx, int ny, int p, double dt, const wf_params* params, i
  * as in wf_set_wind, NULL for rank 0). A new mean wind refactors the slot's
  * operators on the GPU. Clears the slot's guard flag; does not change whether the
  * slot is active. Waits for earlier work on the handle's stream. Errors: WF_EINVAL,
- * WF_ETRUNC, WF_ESINGULAR, WF_ECUDA. */
+ * WF_ETRUNC, WF_ESINGULAR (as wf_set_mean_wind: the slot keeps its wind and its
+ * state), WF_ECUDA. */
 int wf_batch_set_slot(wf_handle* h, int slot, const double* T, const double* fuel, double wind_x, double wind_y,
                       int wind_rank, const double* wind_factors);
 

@@ -920,6 +920,33 @@ int set_slot_wind_factors(wf_handle* h, int slot, int rank, const double* factor
     return WF_OK;
 }
 
+// Mean wind of a slot: its operators are factored for the new one.  A refused wind leaves the slot as it was, with
+// the previous wind's factors built again: the refused ones overwrote them, and neither the handle's launches nor
+// a second request for the same wind may find those.
+int change_wind(wf_handle* h, int slot, double wind_x, double wind_y) {
+    Slot& sl = h->slots[slot];
+    if (sl.wind_x == wind_x && sl.wind_y == wind_y) return WF_OK;
+    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return WF_ECUDA;  // steps in flight use the factors
+    const double old_x = sl.wind_x, old_y = sl.wind_y;
+    sl.wind_x = wind_x;
+    sl.wind_y = wind_y;
+    set_slot_coeffs(h, sl);
+    const int rc = build_factors(h, slot, 1);
+    if (rc != WF_OK) {
+        sl.wind_x = old_x;
+        sl.wind_y = old_y;
+        set_slot_coeffs(h, sl);
+        const int rc2 = build_factors(h, slot, 1);
+        return rc2 == WF_OK ? rc : rc2;
+    }
+    if (h->mms_on && slot == 0) {
+        h->mms.wind_x = wind_x;
+        h->mms.wind_y = wind_y;
+        drop_graphs(h);  // the forcing launch carries the wind by value
+    }
+    return WF_OK;
+}
+
 bool factors_finite(const double* f, size_t n) {
     for (size_t k = 0; k < n; ++k)
         if (!isfinite(f[k])) return false;
@@ -1120,28 +1147,7 @@ int wf_set_wind(wf_handle* h, int rank, const double* factors) {
 
 int wf_set_mean_wind(wf_handle* h, int slot, double wind_x, double wind_y) {
     if (!h || slot < 0 || slot >= h->S || !isfinite(wind_x) || !isfinite(wind_y)) return WF_EINVAL;
-    Slot& sl = h->slots[slot];
-    if (sl.wind_x == wind_x && sl.wind_y == wind_y) return WF_OK;
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return WF_ECUDA;  // steps in flight use the factors
-    const double old_x = sl.wind_x, old_y = sl.wind_y;
-    sl.wind_x = wind_x;
-    sl.wind_y = wind_y;
-    set_slot_coeffs(h, sl);
-    int rc = build_factors(h, slot, 1);
-    if (rc != WF_OK) {
-        // keep the slot usable: back to the previous wind (whose factors were valid)
-        sl.wind_x = old_x;
-        sl.wind_y = old_y;
-        set_slot_coeffs(h, sl);
-        const int rc2 = build_factors(h, slot, 1);
-        return rc2 == WF_OK ? rc : rc2;
-    }
-    if (h->mms_on && slot == 0) {
-        h->mms.wind_x = wind_x;
-        h->mms.wind_y = wind_y;
-        drop_graphs(h);  // the forcing launch carries the wind by value
-    }
-    return WF_OK;
+    return change_wind(h, slot, wind_x, wind_y);
 }
 
 int wf_batch_set_slot(wf_handle* h, int slot, const double* T, const double* fuel, double wind_x, double wind_y,
@@ -1150,15 +1156,9 @@ int wf_batch_set_slot(wf_handle* h, int slot, const double* T, const double* fue
     if (!isfinite(wind_x) || !isfinite(wind_y) || wind_rank < 0 || wind_rank > kMaxRank) return WF_EINVAL;
     if (wind_rank > 0 && (!wind_factors || !factors_finite(wind_factors, 2 * (size_t)wind_rank * (h->Nx + h->Ny))))
         return WF_EINVAL;
-    Slot& sl = h->slots[slot];
-    if (sl.wind_x != wind_x || sl.wind_y != wind_y) {
-        sl.wind_x = wind_x;
-        sl.wind_y = wind_y;
-        set_slot_coeffs(h, sl);
-        const int rc = build_factors(h, slot, 1);
-        if (rc != WF_OK) return rc;
-    }
-    int rc = set_slot_wind_factors(h, slot, wind_rank, wind_factors);
+    int rc = change_wind(h, slot, wind_x, wind_y);
+    if (rc != WF_OK) return rc;
+    rc = set_slot_wind_factors(h, slot, wind_rank, wind_factors);
     if (rc != WF_OK) return rc;
     rc = set_slot_state(h, slot, T, fuel);
     if (rc != WF_OK) return rc;
