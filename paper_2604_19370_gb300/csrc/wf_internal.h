@@ -225,14 +225,16 @@ inline cudaError_t launch_overlapped(void (*kern)(KA...), dim3 grid, unsigned th
 #ifdef __CUDACC__
 // First statement of such a kernel: waits until the kernel before it is complete and its writes are visible.
 // `off` is added to every address the kernel reads, and passes through the wait, so that no load (a read-only one
-// neither) can be moved above it.  A grid of at most kEarlyCtas CTAs then lets the next kernel's CTAs start
+// neither) can be moved above it.  EARLY: a grid of at most kEarlyCtas CTAs then lets the next kernel's CTAs start
 // beside it; larger ones leave that to their end, where the next kernel's CTAs no longer take room from theirs.  us per
 // step, no overlap / at the end / always early: 130^2 13.9 / 13.0 / 12.9, 100 x 64 cubic Strang 37.7 / 36.7 /
 // 35.2, 1026^2 34.8 / 33.9 / 35.6, 8 x 515^2 cubic 105.3 / 104.3 / 107.5.
 constexpr unsigned kEarlyCtas = 2 * 152;
+template <bool EARLY = true>
 __device__ __forceinline__ void grid_wait(long long& off) {
     asm volatile("griddepcontrol.wait;" : "+l"(off)::"memory");
-    if (gridDim.x * gridDim.y * gridDim.z <= kEarlyCtas) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (EARLY && gridDim.x * gridDim.y * gridDim.z <= kEarlyCtas)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 #endif
 

@@ -959,7 +959,7 @@ template <typename P, int PD, int WR, bool XO, int NW>
 __global__ void __launch_bounds__(32 * NW, RowOcc<P, PD>::value) k_quad_rows(const __grid_constant__ QuadArgs<P> a) {
     extern __shared__ __align__(16) unsigned char wind_rows[];
     long long off = (long long)blockIdx.z * a.b.sbytes;
-    grid_wait(off);
+    grid_wait<sizeof(P) == 4>(off);  // (FP64: see even_smem)
     if (!scene_active(a.b)) return;
     using SM = RowsSmem<P, PD, NW>;
     SM& sm = *reinterpret_cast<SM*>(wind_rows);
@@ -967,6 +967,19 @@ __global__ void __launch_bounds__(32 * NW, RowOcc<P, PD>::value) k_quad_rows(con
     const int sg = blockIdx.x / a.ns, strip = a.s0 + (blockIdx.x - sg * a.ns);
     quad_rows<P, PD, WR, XO, NW>(a, off, lane, w, strip * (32 - PD), sg * a.h, sm,
                                  reinterpret_cast<P*>(wind_rows + sizeof(SM)));
+}
+
+// Shared memory a CTA asks for so that `ctas` CTAs spread evenly: no SM holds more than ctas / sms of them, rounded up.
+// The FP64 quadrature is few long CTAs (rounds of element rows on the busiest SM set its time, run_quad).  Started beside the
+// last CTAs of a y pass, they all went to the SMs that were free then, two or three to an SM beside idle
+// ones: 8 x 258^2, PR step 866 us, 377 with this; 64 x 42^2 Strang 885 and 315; 402^2 cubic 514 and 355.
+// Its own CTAs do not let the next kernel start early: x tiles waiting beside them made it slower (8 x 67 x 303 cubic
+// 410 us, 393 without).
+inline size_t even_smem(size_t need, long ctas, int sms) {
+    constexpr size_t per_sm = 228 * 1024, per_cta = 227 * 1024, reserved = 1024;  // of an SM; at most, and by the system, of a CTA
+    const size_t fit = (size_t)((ctas + sms - 1) / sms);
+    const size_t most = per_sm / (fit + 1) / 128 * 128 + 128 - reserved;  // fit + 1 of them are more than an SM holds
+    return most > need && most <= per_cta ? most : need;
 }
 
 template <typename P>
@@ -1059,7 +1072,8 @@ cudaError_t run_quad(const RhsArgs& r, cudaStream_t s) {
         while (hgt > 1 && wind_bytes(hgt) > 48 * 1024) hgt /= 2;
         const int nseg = (r.Ny + hgt - 1) / hgt;
         a.h = threads == 32 ? (r.Ny + nseg - 1) / nseg : hgt;
-        const size_t smem = ring + wind_bytes(a.h);
+        size_t smem = ring + wind_bytes(a.h);
+        if (sizeof(P) == 8) smem = even_smem(smem, strips * nseg, sms);
         if (smem > 24 * 1024) {
             cudaError_t e = allow_dynamic_smem(kern, smem);
             if (e != cudaSuccess) return e;
