@@ -627,7 +627,7 @@ __device__ __forceinline__ void y_mid_tile(const PassArgs<P>& a, const P* band0,
 #pragma unroll
         for (int d = 0; d + 1 < W; ++d) {
             const int r = row0 + d - PD;
-            win[d] = (active && r >= 0 && r < N) ? __ldg(T + r * pitch) : P(0);
+            win[d] = (active && r >= 0 && r < N) ? field_load(T + r * pitch) : P(0);
         }
         P bi[W];  // the rows of B away from the ends of the line
         const bool inner = N > 4 * PD;
@@ -636,8 +636,8 @@ __device__ __forceinline__ void y_mid_tile(const PassArgs<P>& a, const P* band0,
 #pragma unroll
         for (int i = 0; i < M; ++i) {
             const int row = row0 + i, r = row + PD;
-            win[W - 1] = (active && r < N) ? __ldg(T + r * pitch) : P(0);
-            u[i] = (active && row < N) ? __ldg(src + row * pitch) : P(0);
+            win[W - 1] = (active && r < N) ? field_load(T + r * pitch) : P(0);
+            u[i] = (active && row < N) ? field_load(src + row * pitch) : P(0);
             P t = P(0);
             if (inner && row >= 2 * PD && row < N - 2 * PD) {
 #pragma unroll

@@ -350,7 +350,7 @@ __device__ __forceinline__ void quad_strip(const QuadArgs<P>& a, long long off, 
     auto fetch = [&](const P* row, P (&x)[NB]) {
         const P* c = row + shift;
 #pragma unroll
-        for (int k = 0; k < NB; ++k) x[k] = __ldg(c + k);
+        for (int k = 0; k < NB; ++k) x[k] = field_load(c + k);
     };
     auto xcomps = [&](P (&x)[NB], P (&c)[NB]) {
         if (PD > 1 && xb) xe.apply(x);
@@ -695,7 +695,7 @@ __device__ __forceinline__ void quad_rows(const QuadArgs<P>& a, long long off, i
     auto fetch = [&](const P* row, P (&x)[NB]) {
         const P* c = row + shift;
 #pragma unroll
-        for (int k = 0; k < NB; ++k) x[k] = __ldg(c + k);
+        for (int k = 0; k < NB; ++k) x[k] = field_load(c + k);
     };
     auto xcomps = [&](P (&x)[NB], P (&c)[NB]) {
         if (PD > 1 && xb) xe.apply(x);
