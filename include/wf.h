@@ -270,8 +270,8 @@ int wf_launch_count(unsigned long long* n);
  *             that one group's quadrature runs beside the other group's line
  *             passes; the groups join at the end of each wf_step call (and
  *             of each captured graph of steps).  Batches of two or more
- *             slots without manufactured forcing; profiled steps run the
- *             launches of form 1, wf_step_noalloc those of form 0;
+ *             slots without manufactured forcing; elsewhere, and in
+ *             wf_step_noalloc, as 0; profiled steps run the launches of form 1;
  *   shape[7]  slots per group of the persistent step's work order (the order
  *             keeps about two groups' fields live, sized for the L2 cache);
  * 0 selects the built-in rule.

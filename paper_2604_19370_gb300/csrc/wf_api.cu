@@ -588,7 +588,7 @@ int prepare_persist(wf_handle* h) {
     cudaError_t e = persist_step(ph, &plan, false, h->stream);
     if (e == cudaErrorNotSupported) {
         cudaGetLastError();
-        h->tune[6] = 1;  // this handle's arguments do not fit the persistent form
+        h->tune[6] = 0;  // this handle's arguments do not fit the persistent form
         return WF_OK;
     }
     if (e != cudaSuccess) return WF_ECUDA;
@@ -730,10 +730,11 @@ cudaError_t enqueue_step_body(wf_handle* h) {
         return e;
     }
     if (h->prm.scheme == WF_PR && h->prm.F_timing == WF_F_ONCE) {
-        // X_+ lines along x, Y_+ along y.  Step form 1: a launch per array and per kind of strip
+        // X_+ lines along x, Y_+ along y.  Step form 1, and form 3 under profiling: a launch per array and per
+        // kind of strip
         RhsArgs r1 = rhs_args(h, h->Phi, h->R, tau, false);
         const bool pers = use_persist(h) && h->p_ctl;
-        const bool split = h->tune[6] == 1 || (h->tune[6] == 3 && h->gn == 0);
+        const bool split = h->tune[6] == 1 || (h->tune[6] == 3 && h->profiling && h->gn == 0 && !h->noalloc_run);
         r1.parts = split ? 1 : 0;
         if (!quad(S_RHS1, r1)) return e;
         if (pers) {
