@@ -5,9 +5,9 @@ Default workload (one "step" = one Peaceman-Rachford time step of every scenario
 ensemble of 256 scenarios of 256 x 256 elements of quadratic B-splines (258 x 258 = 66,564
 DOFs each, 17.04 M in all), each with a seeded mean wind (direction U[0, 2 pi), speed U[0, 3])
 and ignition point, sharing one seeded fuel field; FP32 bulk with FP64 1-D factorisations; one
-batch handle stepped by the launch form and shapes the autotuner picks (one persistent launch
-per step over every slot, or one launch per pass).  The state (five fields per slot, ~380 MB)
-is larger than the L2 cache, so no flush is needed between steps.  Each rank of a multi-GPU run
+batch handle stepped by the launch form and shapes the autotuner picks (one launch per
+pass, the same over two slot groups, or one persistent launch for the line passes).  The state (four fields
+per slot, ~300 MB) is larger than the L2 cache, so no flush is needed between steps.  Each rank of a multi-GPU run
 steps its own contiguous share of the scenarios (independent problems, no collective).
 
 The same JSON line carries, as extra keys, the single-instance FP64 path on the 1024^2 domain
@@ -59,21 +59,17 @@ def alu_peak(wf, fp64: bool, sm_count: int, mhz: float):
         return sm_count * 128 * 2 * mhz * 1e6 / 1e12, "derived from SM count and clock (probe failed)"
 
 
-def algorithmic_costs(p: int, fused_x2: bool = False) -> dict:
-    """Algorithmic bytes and flops per DOF of each kernel class of a PR step (FP32 values).
+def algorithmic_costs(p: int) -> dict:
+    """Bytes and flops per DOF of the method with basis tables and two substeps (FP32 values).
 
-    Flops count fused multiply-adds (2 flops each) of the sum-factorised method, once per DOF:
-    the quadrature interpolates T, dT/dx (x) and T, dT/dx, dT/dy (y) from p+1 coefficients,
+    A yardstick that does not move with the implementation; the library's step does less (kernel_costs), so no
+    fraction of a pipe is formed from it.  Flops count fused multiply-adds (2 flops each) of the sum-factorised
+    method, once per DOF: the quadrature interpolates T, dT/dx (x) and T, dT/dx, dT/dy (y) from p+1 coefficients,
     2q(p+1) + 3q^2(p+1); the fuel q(p+1) + q^2(p+1); tests them against the basis functions at
     the same cost (the mirror); 6 per Gauss point for the point source; and forms R with two
     Kronecker products, 4W + 1 (W = 2p+1: an x and a y band each, plus the scaled F).  A line
     solve is 4p + 1 per value (p forward, p + 1 backward, 2p spike), + 1 where an increment base
     is added.  Bytes: each field read or written once by its pass.
-
-    These are the method's counts, with basis tables and two substeps, the common yardstick of the rates
-    reported here.  The library's step does less: its quadrature takes 222 multiply-adds a DOF instead of 345
-    (p = 2, monomial components) and stores no F, and Peaceman-Rachford with one F per step is one x and
-    one y pass.
     """
     q = nb = p + 1
     W = 2 * p + 1
@@ -87,19 +83,18 @@ def algorithmic_costs(p: int, fused_x2: bool = False) -> dict:
         "xsolve_1": dict(bytes=16, flops=2 * 2 * line),               # R and Phi in and out
         "ysolve_1": dict(bytes=24, flops=2 * 2 * (line + 1)),         # R, Phi, bases T, phi in; T, phi out
         "matvec_2": dict(bytes=12, flops=2 * mv),                     # T*, F in; R out
-        "xsolve_2": (dict(bytes=12, flops=2 * (mv + line)) if fused_x2 else dict(bytes=8, flops=2 * line)),
+        "xsolve_2": dict(bytes=8, flops=2 * line),
         "ysolve_2": dict(bytes=12, flops=2 * (line + 1)),             # R, base T* in; T out
     }
     step_flops = c["rhs_quadrature_1"]["flops"] + c["xsolve_1"]["flops"] + c["ysolve_1"]["flops"] + \
         2 * mv + 2 * line + c["ysolve_2"]["flops"]
-    # one persistent launch is one whole step: the method's minimum bytes (each pass reads and
-    # writes its fields once, the quadrature's R and Phi consumed by the first x pass: 56 B)
+    # the whole step: the method's minimum bytes (min_step_bytes)
     c["step_persistent"] = dict(bytes=56, flops=step_flops)
     return c
 
 
 def min_step_bytes(scheme: str) -> int:
-    """Least HBM bytes per DOF of one step (FP32): fields read and written once per pass.
+    """Least HBM bytes per DOF of one step of the method (FP32, two substeps): fields read and written once per pass.
 
     PR: x1 reads T, phi and writes its two results and F (20); y1 reads and writes two
     fields (16); x2 reads T*, F and writes its result (12); y2 reads and writes one (8).
@@ -108,6 +103,55 @@ def min_step_bytes(scheme: str) -> int:
     and writes two fields (24).
     """
     return {"pr": 56, "strang": 60, "explicit": 40}[scheme]
+
+
+def quadrature_ops(p: int, rank: int) -> int:
+    """Operations per element of the quadrature kernel away from a fire, a multiply-add, a multiply or an add each.
+
+    On monomial components: of a coefficient row along x and of p+1 columns along y; values and y derivatives at
+    the y points of each x component; T, T_x, T_y at the points; 9 per point, 2 more per rank of the wind variation (as
+    the kernel runs it: 0, 2 or 4); the test sums along x and y, back to rows and added up; and a finished row along x.
+    """
+    q = nb = p + 1
+    comps, value, deriv, sums, flux, scatter = {1: (2, 2, 0, 2, 4, 3), 2: (4, 3, 2, 3, 8, 5), 3: (9, 8, 7, 10, 21, 11)}[p]
+    wr = 0 if rank == 0 else (2 if rank <= 2 else 4)
+    return (comps + nb * comps + nb * (value + deriv) + q * (2 * value + deriv) + q * q * (9 + 2 * wr)
+            + q * (flux + sums) + nb * flux + nb * (scatter + p) + scatter + p + 1)
+
+
+def kernel_costs(p: int, rank: int, scheme: str, split: bool = False) -> dict:
+    """Bytes and flops per DOF and launch of the library's kernels (FP32 values; 2 flops an operation of the FMA pipe).
+
+    Quadrature: T in, R and (first one) Phi out; its reaction, and the fuel it reads for that, run only beside a
+    fire and are left out.  A line pass is 4p + 1 operations per value (each recursion runs twice over a chunk, one
+    scaling) and 1 where a base is added: x reads and writes R and Phi, y reads them and the bases and writes the
+    fields.  The middle y pass of Strang / Crank-Nicolson is two solves and 2p + 1 more for the explicit operator.
+    split: a line pass launches once per array (step form 1).
+    """
+    ops, line = quadrature_ops(p, rank), 4 * p + 1
+    c = {"rhs_quadrature_1": dict(bytes=12, flops=2 * ops), "xsolve_1": dict(bytes=16, flops=2 * 2 * line)}
+    two = dict(bytes=24, flops=2 * 2 * (line + 1))
+    if scheme == "pr":
+        c["ysolve_1"] = two
+        c["step_persistent"] = dict(bytes=40, flops=c["xsolve_1"]["flops"] + two["flops"])
+        if split:
+            for k in ("xsolve_1", "ysolve_1"):
+                c[k] = {q: v // 2 for q, v in c[k].items()}
+    elif scheme == "explicit":
+        c["ysolve_2"] = two
+    else:
+        c["ysolve_y_substep"] = dict(bytes=12, flops=2 * (2 * line + 2 * p + 5))  # R, T in; T** out
+        c["rhs_quadrature_2"] = dict(bytes=8, flops=2 * ops)
+        c["xsolve_2"] = dict(bytes=8, flops=2 * line)
+        c["ysolve_2"] = two
+    return c
+
+
+def step_costs(p: int, rank: int, scheme: str) -> dict:
+    """Bytes and flops per DOF of one step, the sum over its kernels."""
+    c = kernel_costs(p, rank, scheme)
+    c.pop("step_persistent", None)
+    return {q: sum(v[q] for v in c.values()) for q in ("bytes", "flops")}
 
 
 def roofline(kernel: str, ms: float, dofs: int, costs: dict, es: int, hbm_gbs: float, hbm_src: str,
@@ -477,8 +521,11 @@ def run_ensemble(args) -> None:
     status = wf.wf_sync(b.h)
     value, slowest = whole_job_throughput(dofs * args.steps, secs, world, dev)
     ms_per_step = slowest * 1e3 / args.steps
-    # per-kernel device times: the same K steps launched directly, an event pair around each launch
+    # per-kernel device times: the same K steps launched directly, an event pair around each launch (of form
+    # 3, those of form 0, which it launches once per slot group)
     wf.wf_kernel_times(b.h)
+    if tuning[6] == 3:
+        wf.wf_set_tuning(b.h, (*tuning[:6], 0, tuning[7]))
     n0 = wf.wf_launch_count()
     prof_s = timed(True)
     launches = wf.wf_launch_count() - n0
@@ -486,14 +533,13 @@ def run_ensemble(args) -> None:
     peaks = _peaks()
     props = torch.cuda.get_device_properties(dev)
     alu, alu_src = alu_peak(wf, False, props.multi_processor_count, peaks["sm_max_mhz"])
-    costs = algorithmic_costs(first.p)
-    costs["rhs_quadrature_1"]["bytes"] = 16  # no F stored
+    costs = kernel_costs(first.p, first.wind_rank, "pr", split=tuning[6] == 1)
+    per_dof = step_costs(first.p, first.wind_rank, "pr")
     ktab = _kernel_table(kt)
     dom = max(ktab, key=lambda k: ktab[k]["share"])
     workload = f"c4_ensemble_{S_all}x256x256_p2_pr"
     roof = roofline(dom, ktab[dom]["ms_per_launch"], dofs, costs, 4, peaks["hbm_gbs"], peaks["src"], alu, alu_src,
                     _traffic_record(dom, "c4_ensemble_256x256x256_p2_pr") if S_all == 256 else None)
-    step_flops = costs["step_persistent"]["flops"] * dofs
     # the other step forms, timed the same way with the same shapes (the autotuner times every form
     # and keeps the fastest): per-pass launches; one quadrature launch and one persistent launch over
     # every line pass of every slot; the per-pass launches over two slot groups on two streams (form 1, a launch
@@ -558,19 +604,20 @@ def run_ensemble(args) -> None:
         "config": {"workload": workload, "scenarios": S_all, "scenarios_per_rank": S, "nx": 256, "ny": 256,
                    "p": 2, "dofs": S_all * first.dofs, "scheme": "PR",
                    "precision": "fp32 bulk, fp64 1-D factorisation",
-                   "l2": f"state of {S} slots x 5 fields (~{5 * S * 258 * 288 * 4 / 2**20:.0f} MiB) > L2, no flush",
+                   "l2": f"state of {S} slots x 4 fields (~{4 * S * 258 * 288 * 4 / 2**20:.0f} MiB) > L2, no flush",
                    "parallelism": f"scenarios sharded over {world} rank(s), no collective",
                    "launch_shapes": {**{k: v for k, v in zip(wf.TUNING_NAMES, tuning)}, "source": shape_source(args)}},
         "roofline": roof,
-        "step_roofline": {"hbm_frac_of_min_bytes": min_step_bytes("pr") * dofs / (ms_per_step * 1e-3) / 1e9
-                          / peaks["hbm_gbs"],
-                          "alu_frac": step_flops / (ms_per_step * 1e-3) / 1e12 / alu,
-                          "min_bytes_per_dof": min_step_bytes("pr"),
-                          "flops_per_dof": costs["step_persistent"]["flops"]},
+        # of the kernels' own operations and bytes; the method's count beside them
+        "step_roofline": {"hbm_frac": per_dof["bytes"] * dofs / (ms_per_step * 1e-3) / 1e9 / peaks["hbm_gbs"],
+                          "alu_frac": per_dof["flops"] * dofs / (ms_per_step * 1e-3) / 1e12 / alu,
+                          "bytes_per_dof": per_dof["bytes"], "flops_per_dof": per_dof["flops"],
+                          "method_bytes_per_dof": min_step_bytes("pr"),
+                          "method_flops_per_dof": algorithmic_costs(first.p)["step_persistent"]["flops"]},
         "profiled_ms_per_step": prof_s * 1e3 / args.steps,
         "kernels": ktab,
         # the profiled pass launches each kernel once per step over all slots; step form 3 launches
-        # every kernel once per slot group
+        # them once per slot group
         "gpu_launches": launches * (2 if chosen == 3 and S >= 2 else 1),
         "step_form": forms[chosen],
         "other_step_forms": other_forms,
@@ -749,10 +796,8 @@ def run_single(args) -> None:
     peaks = _peaks()
     props = torch.cuda.get_device_properties(dev)
     alu, alu_src = alu_peak(wf, args.fp64, props.multi_processor_count, peaks["sm_max_mhz"])
-    costs = algorithmic_costs(sc.p)
-    costs["rhs_quadrature_1"]["bytes"] = 16  # no F stored
-    if scheme_of(args) == "explicit":
-        costs["ysolve_2"]["bytes"] = 24  # two arrays with their bases
+    costs = kernel_costs(sc.p, sc.wind_rank, scheme_of(args), split=tuning[6] == 1)
+    per_dof = step_costs(sc.p, sc.wind_rank, scheme_of(args))
     ktab = _kernel_table(kt)
     dom = max(ktab, key=lambda k: ktab[k]["share"])
     wname = f"{args.workload}_{sc.nx}x{sc.ny}_p{sc.p}_{scheme_of(args)}"
@@ -769,8 +814,7 @@ def run_single(args) -> None:
                    "launch_shapes": {**{k: v for k, v in zip(wf.TUNING_NAMES, tuning)}, "source": shape_source(args)},
                    "parallelism": f"replicas x{world}"},
         "roofline": roof,
-        "step_hbm_frac": min_step_bytes(scheme_of(args)) * (es / 4) * sc.dofs / (ms_per_step * 1e-3) / 1e9
-        / peaks["hbm_gbs"],
+        "step_hbm_frac": per_dof["bytes"] * (es / 4) * sc.dofs / (ms_per_step * 1e-3) / 1e9 / peaks["hbm_gbs"],
         "profiled_ms_per_step": prof_ms_per_step,
         "kernels": ktab,
         "gpu_launches": launches,
