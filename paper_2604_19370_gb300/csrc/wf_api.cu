@@ -239,7 +239,7 @@ void layout_slot(wf_handle* h, Arena& A) {
         d->tabM = A.take<char>(line_tab_bytes(es, h->p, d->N, h->M));
         d->tabA = A.take<char>(line_tab_bytes(es, h->p, d->N, h->M));
     }
-    if (needs_mid(h)) h->dy.band = A.take<char>((size_t)h->Ny * (2 * h->p + 1) * es);
+    if (needs_mid(h)) h->dy.band = A.take<char>((size_t)h->Ny * (2 * h->p) * es);
     const size_t qx = (size_t)kMaxRank * h->nx * h->q, qy = (size_t)kMaxRank * h->ny * h->q;
     h->mw = A.take<char>(2 * es);
     h->fxq = A.take<char>(qx * es);

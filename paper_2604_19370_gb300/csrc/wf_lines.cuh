@@ -599,11 +599,11 @@ __device__ __forceinline__ void y_tile(const PassArgs<P>& a, long long off, int 
 //   T** = T - (M^y)^{-1} u + Y_+^{-1} (2 u + 2 B T),   B = -theta_y A_y:
 // two solves of one column in one pass instead of a pass for T* and a second one for T**.  T** goes to a
 // field of its own (tiles read the rows of T around theirs).  in: u, base: T, tab: M^y and Y_+, band:
-// rows of B, out: T**.
+// factors of B's rows on differences of T (TabJob), out: T**.
 template <typename P, int PD, int M, bool UNI>
 __device__ __forceinline__ void y_mid_tile(const PassArgs<P>& a, const P* band0, long long off, int cg, int tile,
                                            unsigned char* smem, int tid) {
-    constexpr int W = 2 * PD + 1;
+    constexpr int W = 2 * PD;
     const P* in = shift(a.in[0], off);
     P* out = shift(a.out[0], off);
     const P* base = shift(a.base[0], off);
@@ -623,32 +623,37 @@ __device__ __forceinline__ void y_mid_tile(const PassArgs<P>& a, const P* band0,
     {
         const P* src = in + (active ? line : 0);
         const P* T = base + (active ? line : 0);
-        P win[W];  // T rows i - p .. i + p
+        auto row_of = [&](int r) { return (active && r >= 0 && r < N) ? field_load(T + r * pitch) : P(0); };
+        P dif[W];  // T[i - p + e + 1] - T[i - p + e]
+        P last = row_of(row0 - PD);
 #pragma unroll
-        for (int d = 0; d + 1 < W; ++d) {
-            const int r = row0 + d - PD;
-            win[d] = (active && r >= 0 && r < N) ? field_load(T + r * pitch) : P(0);
+        for (int e = 0; e + 1 < W; ++e) {
+            const P next = row_of(row0 - PD + e + 1);
+            dif[e] = next - last;
+            last = next;
         }
         P bi[W];  // the rows of B away from the ends of the line
         const bool inner = N > 4 * PD;
 #pragma unroll
-        for (int d = 0; d < W; ++d) bi[d] = inner ? __ldg(band + (size_t)(2 * PD) * W + d) : P(0);
+        for (int e = 0; e < W; ++e) bi[e] = inner ? __ldg(band + (size_t)(2 * PD) * W + e) : P(0);
 #pragma unroll
         for (int i = 0; i < M; ++i) {
-            const int row = row0 + i, r = row + PD;
-            win[W - 1] = (active && r < N) ? field_load(T + r * pitch) : P(0);
+            const int row = row0 + i;
+            const P next = row_of(row + PD);
+            dif[W - 1] = next - last;
+            last = next;
             u[i] = (active && row < N) ? field_load(src + row * pitch) : P(0);
             P t = P(0);
             if (inner && row >= 2 * PD && row < N - 2 * PD) {
 #pragma unroll
-                for (int d = 0; d < W; ++d) t += bi[d] * win[d];
+                for (int e = 0; e < W; ++e) t += bi[e] * dif[e];
             } else if (row < N) {
 #pragma unroll
-                for (int d = 0; d < W; ++d) t += __ldg(band + (size_t)row * W + d) * win[d];
+                for (int e = 0; e < W; ++e) t += __ldg(band + (size_t)row * W + e) * dif[e];
             }
             v[i] = P(2) * (u[i] + t);
 #pragma unroll
-            for (int d = 0; d + 1 < W; ++d) win[d] = win[d + 1];
+            for (int e = 0; e + 1 < W; ++e) dif[e] = dif[e + 1];
         }
     }
     const Sweeps<P, PD, M, UNI> sm(shift(a.tab[0], off), kc, C), sy(shift(a.tab[1], off), kc, C);

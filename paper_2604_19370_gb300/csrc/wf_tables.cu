@@ -165,7 +165,13 @@ __global__ void __launch_bounds__(128) k_line_tables(const __grid_constant__ Tab
     }
     if (jb.band) {
         P* b = reinterpret_cast<P*>(out);
-        for (int i = tid; i < N * W; i += blockDim.x) b[i] = (P)entry(i / W, i % W);
+        for (int i = tid; i < N * 2 * PD; i += blockDim.x) {
+            const int r = i / (2 * PD), e = i % (2 * PD), col = r + e - PD;  // factor of T[col + 1] - T[col]
+            double v = 0.0;
+            if (col >= 0 && col + 1 < N)
+                for (int d = e + 1; d < W; ++d) v += entry(r, d);
+            b[i] = (P)v;
+        }
         return;
     }
     constexpr int NV = PD == 1 ? 2 : (PD == 2 ? 4 : 8), D = 2 * PD, EW = 2 * kEndRows;
