@@ -14,6 +14,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <type_traits>
 
 namespace wf {
@@ -197,9 +198,12 @@ cudaError_t launch_lines_p3_f64(int kind, const LineArgs& l, cudaStream_t s);
 // Raise (never lower) the dynamic shared memory a kernel may be launched with.  The limit is a
 // property of the kernel, read when a launch is made; the launches captured in a graph keep the
 // size each needed, so a later, smaller request for the same kernel (another pass, other launch
-// shapes) must not take the limit below them.
+// shapes) must not take the limit below them, nor may one of another thread (another handle) that read the limit
+// before this one raised it.
 template <typename K>
 inline cudaError_t allow_dynamic_smem(K kern, size_t bytes) {
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(kern));
     if (e != cudaSuccess) return e;
