@@ -405,9 +405,8 @@ int wf_batch_capacity(const wf_handle* h);
  * WF_EINVAL.  No counterpart in the paper. */
 int wf_device_bytes(const wf_handle* h, size_t* bytes);
 
-/* Upper bound of the device bytes wf_batch_create would allocate for these
- * arguments (the largest layout over every chunk length the creation may
- * settle on), computed on the host without touching the device: lets a
+/* The device bytes wf_batch_create would allocate for these
+ * arguments, computed on the host without touching the device: lets a
  * caller admit work by memory budget before allocating.  The whole-batch
  * state calls' staging (2 x capacity x Nx x Ny host-type values, allocated
  * on their first use) is not included.  Errors: WF_EINVAL (as

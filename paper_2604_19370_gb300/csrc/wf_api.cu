@@ -10,8 +10,8 @@
 // graph and replayed by wf_step.
 //
 // A handle holds S scenario slots of one grid (S = 1 for wf_create).  Every slot owns
-// one block of device memory with the same layout (fields, wind-dependent operator
-// bands and factors, wind tables, guard flag); kernels address slot z at
+// one block of device memory with the same layout (fields, factor tables of its
+// wind-dependent operators, wind tables, guard flag); kernels address slot z at
 // z * sbytes past slot 0 and skip slots whose active flag is 0, so slots can join and
 // leave between steps without re-capturing the graph.
 #include <limits.h>
@@ -64,7 +64,7 @@ struct Slot {
     double wind_x = 0, wind_y = 0;
     int wind_rank = 0;
     bool active = false;
-    double coef[2][3][3] = {};  // [dir][op][aM, aK, aG]
+    double coef[2][3][3] = {};  // [dir][op][aM, aK, aG], op 0: M, 1: -theta A (y), 2: M + theta A
 };
 
 enum SiteId { S_RHS1, S_X1, S_Y1, S_YMID, S_RHS2, S_X2, S_Y3, S_PERSIST, S_NSITES };
@@ -80,7 +80,7 @@ struct wf_handle {
     wf_params prm;
     Phys phys;
     cudaStream_t own = nullptr, stream = nullptr;
-    // second stream: the quadrature's boundary items run there beside its interior items
+    // second stream: the fuel of a state transfer moves there beside T
     cudaStream_t aux = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     // step form 3: the slots in two groups, the second group's launches on stream gs; while a
@@ -249,19 +249,18 @@ void layout_slot(wf_handle* h, Arena& A) {
 }
 
 // Operator coefficients of a slot for its mean wind:
-//   x: A_x = C_d K + c_W b_x G + c_chi M;  op1 = -theta A_x (band),  op2 = X_+ = M + theta A_x
-//   y: A_y = C_d K + c_W b_y G;            op1 = -theta A_y (band),  op2 = Y_+ = M + theta A_y
+//   x: A_x = C_d K + c_W b_x G + c_chi M;  X_+ = M + theta A_x
+//   y: A_y = C_d K + c_W b_y G;            Y_+ = M + theta A_y, and -theta A_y (the middle pass of Strang's step)
 void set_slot_coeffs(const wf_handle* h, Slot& s) {
     const Phys& c = h->phys;
     const double tau = h->dt;
-    // explicit: the "-theta A" operators carry the full tau (the "+" side is not used)
+    // explicit: only M is solved with
     const bool ex = h->prm.scheme == WF_EXPLICIT;
     const double thx = ex ? tau : (h->prm.scheme == WF_PR ? 0.5 * tau : 0.25 * tau);
     const double thy = ex ? tau : 0.5 * tau;
     double(*x)[3] = s.coef[0];
     double(*y)[3] = s.coef[1];
     x[0][0] = 1.0, x[0][1] = 0.0, x[0][2] = 0.0;
-    x[1][0] = -thx * c.c_chi, x[1][1] = -thx * c.C_d, x[1][2] = -thx * c.c_W * s.wind_x;
     x[2][0] = 1.0 + thx * c.c_chi, x[2][1] = thx * c.C_d, x[2][2] = thx * c.c_W * s.wind_x;
     y[0][0] = 1.0, y[0][1] = 0.0, y[0][2] = 0.0;
     y[1][0] = 0.0, y[1][1] = -thy * c.C_d, y[1][2] = -thy * c.c_W * s.wind_y;

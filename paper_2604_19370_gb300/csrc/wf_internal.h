@@ -65,7 +65,7 @@ struct Phys {
 constexpr int kTabHeader = 64;
 // FP32 takes uniform factors where an operator has them.  FP64 reads every row's factors: its pipe bounds the
 // passes, loads are free beside it, and the end corrections are a tenth to a half more multiply-adds (step, uniform /
-// table: 66^2 quadratic 51.4 / 47.5 us, 8 x 259^2 cubic 890 / 873, 1026^2 690 / 686).
+// table: 66^2 quadratic 53.6 / 48.6 us, 8 x 259^2 cubic 949 / 932, 1026^2 695 / 688).
 template <typename P>
 constexpr bool kUniformFactors = sizeof(P) == 4;
 constexpr int kEndRows = 128;  // J * M at most for the uniform form

@@ -6,8 +6,10 @@ namespace wf {
 namespace {
 
 // Threads of a CTA at most, and CTAs per SM the registers are budgeted for: FP32 with up to 17 values a
-// thread 40 registers (three CTAs; with two, the step of 256 scenarios of 258^2 took 369 us instead of 348), 33
-// values 64 (two; one: 4099^2 cubic 611 instead of 556); FP64 128.
+// thread 40 registers (three CTAs), 33 values 64 (two; one: 4099^2 cubic 611 us instead of 556); FP64 128.
+// The 40 registers are for launches of many waves, and spill (uniform factors, x and y pass: p = 2 72 and 28 bytes with 9
+// values, 96 and 48 with 17; p = 3 36 and 32, 96 and 236).  Step with three / two CTAs: 256 x 258^2 324 / 344 us; launches
+// of one partial wave would rather have two: 1026^2 34.1 / 31.8, 130^2 13.4 / 12.4, 8 x 515^2 cubic 104.3 / 102.7.
 template <typename P, int M>
 struct LineOcc {
     static constexpr int threads = 512;
@@ -37,7 +39,7 @@ __global__ void __launch_bounds__(NT, NT > 512 ? 1 : LineOcc<P, M>::ctas) k_ylin
 
 // The middle pass holds two chunks: FP32 with 17 values 80 registers and tiles of 384 threads, two CTAs per SM, so
 // that the 264 CTAs of a 1026^2 domain run at once (with 512 threads and 128 registers 198 CTAs took two turns of
-// 152: step 79.1 us, now 72.5).
+// 152: step 79.1 us against 72.5; 71.7 since the explicit operator acts on differences).
 template <typename P, int M>
 struct MidOcc {
     static constexpr bool two = sizeof(P) == 4 && M == 17;

@@ -6,7 +6,7 @@
 //   f = u_t - C_d lap u + c_W b.grad u + c_chi u
 //       - [c_chi T_amb + c_rad (T_amb^4 - u^4) + C_nld (u^3 lap u + 3 u^2 |grad u|^2)]
 // at u* (combustion and wind variation off in the study).  k_forcing adds
-// s1 * int f(., t) B_i B_j to one array and s2 * the same to another, by the q-point Gauss
+// s1 * int f(., t) B_i B_j to an array, by the q-point Gauss
 // rule of the load vectors, t read from device memory so that captured graphs stay valid;
 // k_advance_time moves t by one step.  Everything here runs in FP64.
 #include <math.h>

@@ -1098,7 +1098,7 @@ cudaError_t run_quad(const RhsArgs& r, cudaStream_t s) {
     const size_t ring = sizeof(RowsSmem<P, PD, NW>);
     if constexpr (sizeof(P) == 8) {
         // Height by the FP64 pipe: rounds of NW element rows on the busiest SM, fewest first, then the lower
-        // segment (8 x 259^2 cubic, step at height 65 (its rule): 951 us, 1107 at 52, 982 at 33).
+        // segment (8 x 259^2 cubic, step at height 65 (its rule): 932 us, 1096 at 52, 963 at 33).
         int h = r.Ny;
         long best = 0;
         for (int n = 1; n <= r.Ny && strips * (n - 1) < 8L * sms; ++n) {
